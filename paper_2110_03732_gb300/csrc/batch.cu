@@ -89,33 +89,50 @@ __global__ void __launch_bounds__(256) kb_implicit(const ProbStage* __restrict__
 template <typename T> __device__ __forceinline__ const PrimIn<T>& prim_of(const ProbStage& ps);
 template <> __device__ __forceinline__ const PrimIn<double>& prim_of<double>(const ProbStage& ps) { return ps.p64; }
 template <> __device__ __forceinline__ const PrimIn<float>& prim_of<float>(const ProbStage& ps) { return ps.p32; }
-// the D-fluxes in the stencil precision: the FP32 fluxes of the mixed path occupy the
-// first half of the same arrays
-template <typename T> __device__ __forceinline__ FluxOut<T> flux_of(const ProbStage& ps, int d);
-template <> __device__ __forceinline__ FluxOut<double> flux_of<double>(const ProbStage& ps, int d) { return ps.F64[d]; }
-template <> __device__ __forceinline__ FluxOut<float> flux_of<float>(const ProbStage& ps, int d)
+// the D-fluxes of the mixed path: FP32, in the first half of the FP64 arrays
+__device__ __forceinline__ FluxOut<float> flux32_of(const ProbStage& ps, int d)
 {
     FluxOut<float> f;
 #pragma unroll
     for (int v = 0; v < 8; v++) f.p[v] = reinterpret_cast<float*>(ps.F64[d].p[v]);
     return f;
 }
-// item t: kMarch consecutive D-faces (flux_march_item)
+// item t: kMarch consecutive D-faces
+// one item of either precision's face march
 template <int D, bool M, typename T>
-__global__ void __launch_bounds__(256) kb_flux(const ProbStage* __restrict__ P, int s, int stage,
+__device__ __forceinline__ void flux_any_item(const ProbStage& ps, double* sm, long long t)
+{
+    if constexpr (sizeof(T) == 8)
+        flux64_item<M, false, false>(ps.g, D, ps.p64.p, ps.bfs.p, nullptr, ps.psi, ps.alp, ps.F64[D].p, nullptr,
+                                        ps.fe64[D], sm, t);
+    else flux32_item<D, M, false>(ps.g, ps.p32, ps.bfs, ps.psi, ps.alp, flux32_of(ps, D), ps.fe64[D], t);
+}
+
+template <int D, bool M, typename T>
+__global__ void __launch_bounds__(sizeof(T) == 8 ? Flux64<false, false>::NT : 256) kb_flux(const ProbStage* __restrict__ P, int s, int stage,
                                               const Chunk* __restrict__ ch, int nch)
 {
+    __shared__ double sm[sizeof(T) == 8 ? Flux64<false, false>::SM : 1];
     for (int i = blockIdx.x; i < nch; i += gridDim.x) {
         const Chunk k = ch[i];
         const ProbStage& ps = P[k.prob * s + stage];
-        for (long long t = k.begin + threadIdx.x; t < k.end; t += blockDim.x)
-            flux_march_item<D, M, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp, flux_of<T>(ps, D), nullptr,
-                                     ps.fe64[D], t);
+        for (long long t = k.begin + threadIdx.x; t < k.end; t += blockDim.x) flux_any_item<D, M, T>(ps, sm, t);
     }
 }
 
 // item t: kMarch consecutive C-edges along C + 2 when both transverse directions are
-// active (emf_march_item), else one edge (emf_item)
+// active, else one edge (emf_item)
+template <int C, bool M, typename T>
+__device__ __forceinline__ void emf_any_item(const ProbStage& ps, long long t)
+{
+    if (ps.g.act[(C + 1) % 3] && ps.g.act[(C + 2) % 3]) {
+        if constexpr (sizeof(T) == 8) emf64_item<M, false>(ps.g, C, ps.p64.p, ps.bfs.p, ps.psi, ps.alp, ps.Eh64[C], t);
+        else emf_march_item<C, M, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp, ps.Eh64[C], t);
+    } else {
+        emf_item<C, M, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp, ps.Eh64[C], t);
+    }
+}
+
 template <int C, bool M, typename T>
 __global__ void __launch_bounds__(256) kb_emf(const ProbStage* __restrict__ P, int s, int stage,
                                              const Chunk* __restrict__ ch, int nch)
@@ -123,11 +140,7 @@ __global__ void __launch_bounds__(256) kb_emf(const ProbStage* __restrict__ P, i
     for (int i = blockIdx.x; i < nch; i += gridDim.x) {
         const Chunk k = ch[i];
         const ProbStage& ps = P[k.prob * s + stage];
-        const bool march = ps.g.act[(C + 1) % 3] && ps.g.act[(C + 2) % 3];
-        for (long long t = k.begin + threadIdx.x; t < k.end; t += blockDim.x) {
-            if (march) emf_march_item<C, M, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp, ps.Eh64[C], t);
-            else emf_item<C, M, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp, ps.Eh64[C], t);
-        }
+        for (long long t = k.begin + threadIdx.x; t < k.end; t += blockDim.x) emf_any_item<C, M, T>(ps, t);
     }
 }
 
@@ -217,15 +230,6 @@ struct PersistLists {
         }                                                                               \
     }
 
-template <int C, bool M, typename T>
-__device__ __forceinline__ void emf_any_item(const ProbStage& ps, long long t)
-{
-    if (ps.g.act[(C + 1) % 3] && ps.g.act[(C + 2) % 3])
-        emf_march_item<C, M, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp, ps.Eh64[C], t);
-    else
-        emf_item<C, M, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp, ps.Eh64[C], t);
-}
-
 // nsteps IMEX steps of every problem: per stage the implicit solves, then the face
 // fluxes and edge EMFs (which read the same stage primitives and write separate
 // arrays), then the update, with a grid barrier after each phase; FIXED-boundary
@@ -242,6 +246,7 @@ __global__ void __launch_bounds__(128, (sizeof(T) == 4 ? 4 : 2)) kb_persistent(c
                                                      BarrierState* bs, int nsteps, unsigned long long limit_ns,
                                                      int any_fixed)
 {
+    __shared__ double sm[sizeof(T) == 8 ? Flux64<false, false>::SM : 1];
     const unsigned nb = gridDim.x;
     for (int step = 0; step < nsteps; step++) {
         if (any_fixed) {
@@ -264,18 +269,12 @@ __global__ void __launch_bounds__(128, (sizeof(T) == 4 ? 4 : 2)) kb_persistent(c
             PERSIST_ITEMS(WL_IMP, 0, (implicit_item<false, false, sizeof(T) == 4>(ps.g, ps.imp, t)))
             PERSIST_ITEMS(WL_IMP, 1, (implicit_item<true, false, sizeof(T) == 4>(ps.g, ps.imp, t)))
             if (!grid_barrier(bs, nb, limit_ns)) return;
-            PERSIST_ITEMS(WL_FLUX + 0, 0, (flux_march_item<0, false, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp,
-                                                                       flux_of<T>(ps, 0), nullptr, ps.fe64[0], t)))
-            PERSIST_ITEMS(WL_FLUX + 0, 1, (flux_march_item<0, true, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp,
-                                                                      flux_of<T>(ps, 0), nullptr, ps.fe64[0], t)))
-            PERSIST_ITEMS(WL_FLUX + 1, 0, (flux_march_item<1, false, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp,
-                                                                       flux_of<T>(ps, 1), nullptr, ps.fe64[1], t)))
-            PERSIST_ITEMS(WL_FLUX + 1, 1, (flux_march_item<1, true, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp,
-                                                                      flux_of<T>(ps, 1), nullptr, ps.fe64[1], t)))
-            PERSIST_ITEMS(WL_FLUX + 2, 0, (flux_march_item<2, false, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp,
-                                                                       flux_of<T>(ps, 2), nullptr, ps.fe64[2], t)))
-            PERSIST_ITEMS(WL_FLUX + 2, 1, (flux_march_item<2, true, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp,
-                                                                      flux_of<T>(ps, 2), nullptr, ps.fe64[2], t)))
+            PERSIST_ITEMS(WL_FLUX + 0, 0, (flux_any_item<0, false, T>(ps, sm, t)))
+            PERSIST_ITEMS(WL_FLUX + 0, 1, (flux_any_item<0, true, T>(ps, sm, t)))
+            PERSIST_ITEMS(WL_FLUX + 1, 0, (flux_any_item<1, false, T>(ps, sm, t)))
+            PERSIST_ITEMS(WL_FLUX + 1, 1, (flux_any_item<1, true, T>(ps, sm, t)))
+            PERSIST_ITEMS(WL_FLUX + 2, 0, (flux_any_item<2, false, T>(ps, sm, t)))
+            PERSIST_ITEMS(WL_FLUX + 2, 1, (flux_any_item<2, true, T>(ps, sm, t)))
             PERSIST_ITEMS(WL_EMF + 0, 0, (emf_any_item<0, false, T>(ps, t)))
             PERSIST_ITEMS(WL_EMF + 0, 1, (emf_any_item<0, true, T>(ps, t)))
             PERSIST_ITEMS(WL_EMF + 1, 0, (emf_any_item<1, false, T>(ps, t)))
@@ -436,7 +435,9 @@ cudaError_t launch_stage(grmhd_batch* b, int stage, cudaStream_t st, unsigned ma
             const int kind = WL_FLUX + d;
             if (!(mask >> kind & 1u) || !b->cnt[kind][m]) continue;
             const Chunk* ch = b->d_chunks + b->off[kind][m];
-            const int nch = b->cnt[kind][m], th = b->cfg[kind].threads, gr = grid_of(b, kind, m);
+            // (the FP64 fluxes' shared memory is laid out for this many threads at most)
+            const int nch = b->cnt[kind][m], gr = grid_of(b, kind, m);
+            const int th = b->mixed ? b->cfg[kind].threads : std::min(b->cfg[kind].threads, Flux64<false, false>::NT);
 #define KB_FLUX(DD, MM)                                                                 \
     if (b->mixed) kb_flux<DD, MM, float><<<gr, th, 0, st>>>(P, s, stage, ch, nch); \
     else kb_flux<DD, MM, double><<<gr, th, 0, st>>>(P, s, stage, ch, nch);

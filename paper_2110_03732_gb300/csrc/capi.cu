@@ -943,7 +943,9 @@ grmhd_status grmhd_bounds_violations(long long* count, int reset)
 #ifdef GRMHD_CHECK_BOUNDS
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(e, "synchronise before reading the bounds counters");
-    unsigned long long (*const readers[])(bool) = {oob_kernels, oob_glm, oob_elliptic, oob_batch, oob_noalloc};
+    unsigned long long (*const readers[])(bool) = {oob_kernels, oob_implicit, oob_flux, oob_stencil64, oob_stencil64m,
+                                                      oob_stencil64p, oob_stencil64mp, oob_stencil32, oob_glm, oob_elliptic,
+                                                      oob_batch, oob_noalloc};
     unsigned long long total = 0;
     for (auto rd : readers) {
         const unsigned long long v = rd(reset != 0);

@@ -25,122 +25,17 @@
 
 namespace grmhd {
 
-// HLL fluxes of the 12 variables at the D-face with padded coordinates c (between the
-// cells of linear indices rm and r0 = c - e_D, c) from the reconstructed states:
-// prL / prR the 8 primitives, BL / BR the coordinate B = q_B / psi^6, phL / phR
-// Phi = q_Phi / psi^6.  Writes twice the flux (the update folds the 1/2).
-template <int D, bool M>
-__device__ __forceinline__ void glm_face_flux(const Dims& g, const GlmFluxArgs& a, long long rm, long long r0,
-                                              const double* prL, const double* prR, const double* BL,
-                                              const double* BR, double phL, double phR)
-{
-    const double* __restrict__ psi = M ? a.psi : nullptr;
-    const double* __restrict__ alp = M ? a.alp : nullptr;
-    constexpr int D1 = (D + 1) % 3, D2 = (D + 2) % 3;
-    const double psf = psi ? 0.5 * (psi[rm] + psi[r0]) : 1.0;
-    const double alf = alp ? 0.5 * (alp[rm] + alp[r0]) : 1.0;
-    const double pf2 = psf * psf, pf4 = pf2 * pf2, pf6 = pf4 * pf2;
-    FaceState sL, sR;
-    face_state<double>(prL, BL, D, psf, alf, g.gh, sL);
-    face_state<double>(prR, BR, D, psf, alf, g.gh, sR);
-    // HLL with c+ = c- = alpha sqrt(gamma^DD) (Sec. 2.5, maximal diffusivity); with equal
-    // speeds (c f_L + c f_R - c^2 (q_R - q_L)) / 2c = (f_L + f_R - c (q_R - q_L)) / 2
-    const double cs = psi ? alf * rcp_pos(pf2) : alf;
-    const long long o = r0;
-#pragma unroll
-    for (int v = 0; v < 8; v++) a.F[v][o] = sL.f[v] + sR.f[v] - cs * (sR.q[v] - sL.q[v]);
-    // q_B^j = psi^6 B^j with (f_B^j)^D = eta^{jDk} alpha psi^4 E^k: 0, -alpha psi^4 E^D2,
-    // +alpha psi^4 E^D1 for j = D, D1, D2; q_Phi = psi^6 Phi with (f_Phi)^D = alpha q_B^D
-    const double ap4 = alf * pf4;
-    double qL[4], qR[4], fL[4], fR[4];
-    qL[D] = pf6 * BL[D];
-    qR[D] = pf6 * BR[D];
-    fL[D] = 0.0;
-    fR[D] = 0.0;
-    qL[D1] = pf6 * BL[D1];
-    qR[D1] = pf6 * BR[D1];
-    fL[D1] = -ap4 * prL[5 + D2];
-    fR[D1] = -ap4 * prR[5 + D2];
-    qL[D2] = pf6 * BL[D2];
-    qR[D2] = pf6 * BR[D2];
-    fL[D2] = ap4 * prL[5 + D1];
-    fR[D2] = ap4 * prR[5 + D1];
-    qL[3] = pf6 * phL;
-    qR[3] = pf6 * phR;
-    fL[3] = alf * qL[D];
-    fR[3] = alf * qR[D];
-#pragma unroll
-    for (int v = 0; v < 4; v++) a.F[8 + v][o] = fL[v] + fR[v] - cs * (qR[v] - qL[v]);
-}
-
-// MC (or PPM when P) reconstruction of the 8 primitives, B^i = q_B^i / psi^6 and
-// Phi = q_Phi / psi^6 to K consecutive D-faces per thread, marched along D with one
-// LineRec per quantity (as flux_march_item)
-template <int D, bool M, bool P>
-__device__ __forceinline__ void glm_flux_march_item(const Dims& g, const GlmFluxArgs& a, long long t)
-{
-    using Rec = LineRec<double, P>;
-    const double* __restrict__ psi = M ? a.psi : nullptr;
-    constexpr int NV = 12;
-    int c[3], f0, f1;
-    march_coords<D>(g, t, c, f0, f1);
-    auto load = [&](int m, double* x) {
-        int cs[3] = {c[0], c[1], c[2]};
-        cs[D] = P ? ext_cell(g, D, m) : m;
-        const long long mi = cell_at(g, cs);
-#pragma unroll
-        for (int v = 0; v < 8; v++) x[v] = a.prim[v][mi];
-        double ip6 = 1.0;
-        if (psi) {
-            const double ps = psi[lin(g, cs[0], cs[1], cs[2])], p2 = ps * ps;
-            ip6 = rcp_pos(p2 * p2 * p2);
-        }
-#pragma unroll
-        for (int e = 0; e < 3; e++) x[8 + e] = a.qB[e][mi] * ip6;
-        x[11] = a.qphi[mi] * ip6;
-    };
-    Rec rec[NV];
-    {
-        double w[Rec::NINIT][NV];
-#pragma unroll
-        for (int k = 0; k < Rec::NINIT; k++) load(f0 - Rec::NINIT + Rec::AHEAD + k, w[k]);
-#pragma unroll
-        for (int v = 0; v < NV; v++) {
-            double x[Rec::NINIT];
-#pragma unroll
-            for (int k = 0; k < Rec::NINIT; k++) x[k] = w[k][v];
-            rec[v].init(x);
-        }
-    }
-    int cm[3] = {c[0], c[1], c[2]};
-    cm[D] = f0 - 1;
-    long long rm = lin(g, cm[0], cm[1], cm[2]);
-    for (int f = f0; f < f1; f++) {
-        double x[NV];
-        load(f + Rec::AHEAD, x);
-        double prL[8], prR[8], BL[3], BR[3], phL, phR;
-#pragma unroll
-        for (int v = 0; v < 8; v++) rec[v].step(x[v], prL[v], prR[v]);
-#pragma unroll
-        for (int e = 0; e < 3; e++) rec[8 + e].step(x[8 + e], BL[e], BR[e]);
-        rec[11].step(x[11], phL, phR);
-        c[D] = f;
-        const long long r0 = lin(g, c[0], c[1], c[2]);
-        glm_face_flux<D, M>(g, a, rm, r0, prL, prR, BL, BR, phL, phR);
-        rm = r0;
-    }
-}
-
 template <int D, bool M, bool P = false>
-__global__ void __launch_bounds__(128) k_glm_flux(Dims g, GlmFluxArgs a)
+__global__ void __launch_bounds__(Flux64<P, true>::NT, 4) k_glm_flux(Dims g, GlmFluxArgs a)
 {
+    __shared__ double sm[Flux64<P, true>::SM];
     grid_dep_sync();
     const long long nq = g.dq[D].d;   // chunks of g.mk[D] faces per line
     const long long tot = nq * (D == 0 ? (long long)g.n[1] * g.n[2]
                                        : (D == 1 ? (long long)g.n[0] * g.n[2] : (long long)g.n[0] * g.n[1]));
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot;
          t += (long long)gridDim.x * blockDim.x)
-        glm_flux_march_item<D, M, P>(g, a, t);
+        flux64_item<M, P, true>(g, D, a.prim, a.qB, a.qphi, a.psi, a.alp, a.F, nullptr, nullptr, sm, t);
 }
 
 __device__ __forceinline__ void glm_out(const GlmUpdateArgs& a, int v, long long o, double L, bool has_r)
@@ -238,29 +133,23 @@ static int glm_grid(long long work, int threads, int nsm)
     return (int)b;
 }
 
-template <int D, bool M, bool P>
-static int glm_blocks_per_sm()
-{
-    static int nb = 0;
-    if (nb < 1) {
-        int q = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_glm_flux<D, M, P>, 128, 0) != cudaSuccess || q < 1)
-            q = 1;
-        nb = q;
-    }
-    return nb;
-}
-
 // faces per thread as for the staggered-field flux kernels
 template <int D, bool M, bool P>
 static void glm_flux_launch(const Dims& g, const GlmFluxArgs& a, int nsm, cudaStream_t st)
 {
+    constexpr int NT = Flux64<P, true>::NT;
     const long long other = D == 0 ? (long long)g.n[1] * g.n[2]
                                    : (D == 1 ? (long long)g.n[0] * g.n[2] : (long long)g.n[0] * g.n[1]);
-    const int K = march_len(g.n[D], other, nsm, glm_blocks_per_sm<D, M, P>(), P ? 1.0 : 0.6);
+    static int nb_sm = 0;   // resident blocks per SM, queried once
+    if (nb_sm < 1) {
+        int q = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_glm_flux<D, M, P>, NT, 0) != cudaSuccess || q < 1)
+            q = 1;
+        nb_sm = q;
+    }
     Dims gl = g;
-    set_march(gl, D, K);
-    launch_k(k_glm_flux<D, M, P>, glm_grid((long long)gl.dq[D].d * other, 128, nsm), 128, st, gl, a);
+    set_march(gl, D, march_len(g.n[D], other, nsm, nb_sm, P ? 1.0 : 0.6, NT));
+    launch_k(k_glm_flux<D, M, P>, glm_grid((long long)gl.dq[D].d * other, NT, nsm), NT, st, gl, a);
 }
 
 template <bool P>

@@ -12,6 +12,7 @@
 #include <stdint.h>
 
 #include "dword.cuh"
+#include "fixrec.cuh"
 
 namespace grmhd {
 
@@ -309,13 +310,31 @@ __device__ __forceinline__ T minmod3(T a, T b, T c)
     return ((ia ^ ib) | (ia ^ ic)) < 0 ? T(0) : Bits<T>::from(r);
 }
 
-// left/right states at the face between a1 and a2 from the four cells a0 a1 a2 a3
+// the same by the FP64 sequence: edge states of cell b
+__device__ __forceinline__ void mc_cell_f64(double a, double b, double x, double& lo, double& hi)
+{
+    const double h = minmod3<double>(b - a, scale_pow2<double, -2>(x - a), x - b);
+    lo = b - h;
+    hi = b + h;
+}
+
+// left/right states at the face between a1 and a2 from the four cells a0 a1 a2 a3 (FP64:
+// fixed point, fixrec.cuh)
 template <typename T>
 __device__ __forceinline__ void mc_face(T a0, T a1, T a2, T a3, T& L, T& R)
 {
-    const T dm = a1 - a0, d0 = a2 - a1, dp = a3 - a2;
-    L = a1 + minmod3<T>(dm, scale_pow2<T, -2>(a2 - a0), d0);
-    R = a2 - minmod3<T>(d0, scale_pow2<T, -2>(a3 - a1), dp);
+    if constexpr (sizeof(T) == 8) {
+        double o;
+        const bool l = fx_mc_cell(a0, a1, a2, o, L), r = fx_mc_cell(a1, a2, a3, R, o);
+        if (!(l && r)) {
+            mc_cell_f64(a0, a1, a2, o, L);
+            mc_cell_f64(a1, a2, a3, R, o);
+        }
+    } else {
+        const T dm = a1 - a0, d0 = a2 - a1, dp = a3 - a2;
+        L = a1 + minmod3<T>(dm, scale_pow2<T, -2>(a2 - a0), d0);
+        R = a2 - minmod3<T>(d0, scale_pow2<T, -2>(a3 - a1), dp);
+    }
 }
 
 // 1/sqrt(x) through CUDA's reciprocal square root, in the precision of x (for the
@@ -391,6 +410,25 @@ __device__ __forceinline__ void ppm_limit(T a0, T& aL, T& aR)
 template <typename T>
 __device__ __forceinline__ void ppm_face(const T* a, T& L, T& R)
 {
+    if constexpr (sizeof(T) == 8) {
+        const unsigned E = fx_max(fx_block(a[0], a[1], a[2]), fx_block(a[3], a[4], a[5]));
+        bool near = fx_finite(E);
+        for (int k = 0; k < 6; k++) near = near && fx_near(a[k], E);
+        if (near) {
+            long long x[6], s[6], f[3];
+            for (int k = 0; k < 6; k++) x[k] = fx_of(a[k], E);
+            for (int k = 1; k < 5; k++) s[k] = 2 * fx_half_slope(x[k - 1], x[k], x[k + 1]);
+            for (int k = 0; k < 3; k++) f[k] = fx_iface(x[k + 1], x[k + 2], s[k + 1], s[k + 2]);
+            long long l = f[0], r = f[1];
+            fx_limit(x[2], l, r);
+            L = fx_to(r, E);
+            l = f[1];
+            r = f[2];
+            fx_limit(x[3], l, r);
+            R = fx_to(l, E);
+            return;
+        }
+    }
     const T im = ppm_iface<T>(a[0], a[1], a[2], a[3]);
     const T i0 = ppm_iface<T>(a[1], a[2], a[3], a[4]);
     const T ip = ppm_iface<T>(a[2], a[3], a[4], a[5]);

@@ -150,18 +150,11 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
 // face fluxes (Sec. 2.1, Sec. 2.5, Sec. 5 defaults): item t = D-face t
 // ---------------------------------------------------------------------------
 
-// cell-centred densitised q_B^e of the (mapped) cell: from the staggered faces on
-// the FP64 path, from the stage's FP32 copy on the mixed path
-__device__ __forceinline__ double cell_qB_in(const Dims& g, const PrimIn<double>&, const CP3& bf, int e, const int* cs,
-                                             long long)
-{
-    return cell_qB(g, bf.p[e], e, cs);
-}
-__device__ __forceinline__ float cell_qB_in(const Dims&, const PrimIn<float>& pa, const CP3&, int e, const int*,
-                                            long long mi)
-{
-    return pa.p[8 + e][mi];
-}
+// a sign passed as a type
+template <int S>
+struct SignConst {
+    static constexpr int value = S;
+};
 
 // the upwind edge EMF of Sec. 3.2 (Londrillo & Del Zanna 2004) with c+ = c- in each
 // direction, where the four-state weights are all 1/4 and the diffusive coefficients
@@ -176,9 +169,8 @@ __device__ __forceinline__ T uct_edge(T hLL, T hLR, T hRL, T hRR, T ca, T cb, T 
 // HLL flux at the D-face with padded coordinates c (between the cells of linear
 // indices rm = c - e_D and r0 = c) from the reconstructed states: prL / prR the 8
 // primitives (coordinate u^i and E^i), BL / BR the coordinate B with the two transverse
-// components set (the normal one is the face's own).  Writes twice the flux at r0, and
-// the ideal-limit transport velocities when vbar is set.  prL, prR, BL, BR are
-// overwritten.
+// components set (the normal one is the face's own).  Writes twice the flux at r0.  prL,
+// prR, BL, BR are overwritten.  FP32 (mixed precision).
 //
 // Eh (flat metric only, else NULL): Eh[C] set for an edge direction C != D whose
 // third direction is inactive (a 1-D or 2-D grid).  Its edges then coincide with the
@@ -186,11 +178,12 @@ __device__ __forceinline__ T uct_edge(T hLL, T hLR, T hRL, T hRR, T ca, T cb, T 
 // transverse q_B, which are this face's states: the face writes hat{E}_C, what emf_item
 // computes from the same MC or PPM values (to round-off: the edge formula here is
 // reduced for the coinciding states).
-template <int D, bool M, typename T>
-__device__ __forceinline__ void face_flux(const Dims& g, const CP3& bf, const double* psi_in, const double* alp_in,
-                                          const int* c, long long rm, long long r0, T* prL, T* prR, T* BL, T* BR,
-                                          const FluxOut<T>& F, double* const* vbar, double* const* Eh = nullptr)
+template <int D, bool M>
+__device__ __forceinline__ void face_flux32(const Dims& g, const CP3& bf, const double* psi_in, const double* alp_in,
+                                            const int* c, long long rm, long long r0, float* prL, float* prR,
+                                            float* BL, float* BR, const FluxOut<float>& F, double* const* Eh)
 {
+    using T = float;
     const double* __restrict__ psi = M ? psi_in : nullptr;
     const double* __restrict__ alp = M ? alp_in : nullptr;
     constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
@@ -238,44 +231,48 @@ __device__ __forceinline__ void face_flux(const Dims& g, const CP3& bf, const do
         const T hv = v == 0 || v == 4 ? h4 : (v < 4 ? h6 : h2);
         F.p[v][o] = (gL[v] + gR[v]) * hv;
     }
-    if (vbar && vbar[0]) {
-        // App. A steps (i)-(ii): vhat^j = alpha v^j (beta = 0) of the L and R states,
-        // vbar^j = (c- vhat^j_R + c+ vhat^j_L)/(c- + c+), their mean for c+ = c-;
-        // v^j = u_hat^j / (psi^2 W)
-        const double al = (double)(alf * ipf2);
-        const double iL = (double)iWL, iR = (double)iWR;
-        const double vL1 = al * (double)prL[1 + T1] * iL, vR1 = al * (double)prR[1 + T1] * iR;
-        const double vL2 = al * (double)prL[1 + T2] * iL, vR2 = al * (double)prR[1 + T2] * iR;
-        vbar[0][o] = (vR1 + vL1) * 0.5;
-        vbar[1][o] = (vR2 + vL2) * 0.5;
-    }
 }
 
 // Marching reconstruction along a line of cells, one quantity: the face states of the
-// faces f0, f0+1, ... from one new cell per face.  MC keeps the last two cell values,
-// their difference and the older cell's right-face state; PPM keeps the last two cell
-// values, the newer one's MC slope, the interface value below it and the limited right
-// edge of the cell before.  Each step returns the states of face f (between cells f-1
-// and f): bitwise those of mc_face / ppm_face, whose slopes and interface values are
-// the same expressions, each now evaluated once.
+// faces f0, f0+1, ... from one new cell per face.  MC keeps the last two cell values
+// (FP32 also their difference) and the older cell's right-face state; PPM keeps the last
+// two cell values, the newer one's MC slope, the interface value below it and the limited
+// right edge of the cell before.  step() at face f takes cell f + AHEAD and returns the
+// states of that face (between cells f-1 and f): in FP32 bitwise those of mc_face /
+// ppm_face, whose slopes and interface values are the same expressions, each now
+// evaluated once; in FP64 by fixed point (fixrec.cuh), MC's states as mc_face rounds
+// them.  A march pushes the two cells before the one that step() takes at face
+// f0 - WARM; the states of its WARM first steps are not valid yet.
 template <typename T, bool P>
 struct LineRec;
 
-template <typename T>
-struct LineRec<T, false> {
-    static constexpr int NINIT = 3, AHEAD = 1;   // cells f0-2..f0 first; step f loads f+1
-    T a, b, d, l;
-    __device__ __forceinline__ void init(const T* x)
+template <>
+struct LineRec<double, false> {
+    static constexpr int WARM = 1, AHEAD = 1;
+    double a, b, l;
+    __device__ __forceinline__ void push(double x)
     {
-        a = x[1];
-        b = x[2];
-        d = b - a;
-        l = a + minmod3<T>(a - x[0], scale_pow2<T, -2>(b - x[0]), d);
+        a = b;
+        b = x;
+        l = 0.0;
     }
-    __device__ __forceinline__ void step(T x, T& L, T& R)
+};
+
+template <>
+struct LineRec<float, false> {
+    static constexpr int WARM = 1, AHEAD = 1;
+    float a, b, d, l;
+    __device__ __forceinline__ void push(float x)
     {
-        const T dn = x - b;
-        const T hs = minmod3<T>(d, scale_pow2<T, -2>(x - a), dn);
+        a = b;
+        b = x;
+        d = b - a;
+        l = 0.0f;
+    }
+    __device__ __forceinline__ void step(float x, float& L, float& R)
+    {
+        const float dn = x - b;
+        const float hs = minmod3<float>(d, scale_pow2<float, -2>(x - a), dn);
         L = l;
         R = b - hs;
         l = b + hs;
@@ -285,38 +282,74 @@ struct LineRec<T, false> {
     }
 };
 
+// PPM at cell a0 by the FP64 (or FP32) sequence: fx_ppm_cell's outputs
+template <typename T>
+__device__ __forceinline__ void ppm_cell(T a0, T a1, T x, T s0, T ip, T& lo, T& hi, T& in, T& s1)
+{
+    s1 = ppm_slope<T>(a0, a1, x);
+    in = ppm_iface_s<T>(a0, a1, s0, s1);
+    lo = ip;
+    hi = in;
+    ppm_limit<T>(a0, lo, hi);
+}
+
 template <typename T>
 struct LineRec<T, true> {
-    static constexpr int NINIT = 5, AHEAD = 2;   // cells f0-3..f0+1 first; step f loads f+2
-    T a0, a1, s0, ip, lr;                        // a_f, a_f+1, slope_f, I_f-1/2, right edge_f-1
-    __device__ __forceinline__ void init(const T* x)
+    static constexpr int WARM = 3, AHEAD = 2;
+    T a0, a1, s0, ip, lr;   // a_f, a_f+1, slope_f, I_f-1/2, right edge_f-1
+    __device__ __forceinline__ void push(T x)
     {
-        const T sm2 = ppm_slope<T>(x[0], x[1], x[2]);
-        const T sm1 = ppm_slope<T>(x[1], x[2], x[3]);
-        s0 = ppm_slope<T>(x[2], x[3], x[4]);
-        T lL = ppm_iface_s<T>(x[1], x[2], sm2, sm1);
-        ip = ppm_iface_s<T>(x[2], x[3], sm1, s0);
-        T lR = ip;
-        ppm_limit<T>(x[2], lL, lR);
-        lr = lR;
-        a0 = x[3];
-        a1 = x[4];
+        a0 = a1;
+        a1 = x;
+        s0 = T(0);
+        ip = a0;
+        lr = a0;
     }
     __device__ __forceinline__ void step(T x, T& L, T& R)
     {
-        const T s1 = ppm_slope<T>(a0, a1, x);
-        const T in = ppm_iface_s<T>(a0, a1, s0, s1);
-        T rL = ip, rR = in;
-        ppm_limit<T>(a0, rL, rR);
+        T hi, in, s1;
         L = lr;
-        R = rL;
-        lr = rR;
+        bool done = false;
+        if constexpr (sizeof(T) == 8) done = fx_ppm_cell(a0, a1, x, s0, ip, R, hi, in, s1);
+        if (!done) ppm_cell<T>(a0, a1, x, s0, ip, R, hi, in, s1);
+        lr = hi;
         ip = in;
         s0 = s1;
         a0 = a1;
         a1 = x;
     }
 };
+
+// one step of N marches: the states L, R at a face from the new values x.  FP64 MC runs
+// the N fixed-point cells without a branch between them (their integer chains interleave)
+// and then redoes by the FP64 sequence the ones that need it, if any do.
+template <int N, typename T, bool P>
+__device__ __forceinline__ void line_step(LineRec<T, P>* rec, const T* x, T* L, T* R)
+{
+    if constexpr (sizeof(T) == 8 && !P) {
+        unsigned redo = 0;
+        double l[N];
+#pragma unroll
+        for (int v = 0; v < N; v++) {
+            L[v] = rec[v].l;
+            if (!fx_mc_cell(rec[v].a, rec[v].b, x[v], R[v], l[v])) redo |= 1u << v;
+        }
+        if (redo) {
+#pragma unroll
+            for (int v = 0; v < N; v++)
+                if (redo >> v & 1u) mc_cell_f64(rec[v].a, rec[v].b, x[v], R[v], l[v]);
+        }
+#pragma unroll
+        for (int v = 0; v < N; v++) {
+            rec[v].l = l[v];
+            rec[v].a = rec[v].b;
+            rec[v].b = x[v];
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < N; v++) rec[v].step(x[v], L[v], R[v]);
+    }
+}
 
 // item t of a face march along D in chunks of K: the padded coordinates c of the
 // line (c[D] unset) and its faces f0 .. f1-1 (padded indices).  Chunks along D,
@@ -340,12 +373,13 @@ __device__ __forceinline__ void march_coords(const Dims& g, long long t, int* c,
 // one cell and reconstructs once (the per-face forms load four or six cells and
 // compute two MC slopes, or three interface values and two parabola limits).  Items:
 // chunks of K faces along D, x-fastest over the other directions (for D = 0 the chunks
-// themselves run along x).
-template <int D, bool M, typename T, bool P = false>
-__device__ __forceinline__ void flux_march_item(const Dims& g, const PrimIn<T>& prim, const CP3& bf,
-                                                const double* psi_in, const double* alp_in, const FluxOut<T>& F,
-                                                double* const* vbar, double* const* Eh, long long t)
+// themselves run along x).  FP32 (mixed precision); FP64 is flux64_item.
+template <int D, bool M, bool P>
+__device__ __forceinline__ void flux32_item(const Dims& g, const PrimIn<float>& prim, const CP3& bf,
+                                            const double* psi_in, const double* alp_in, const FluxOut<float>& F,
+                                            double* const* Eh, long long t)
 {
+    using T = float;
     using Rec = LineRec<T, P>;
     const double* __restrict__ psi = M ? psi_in : nullptr;
     constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
@@ -365,37 +399,329 @@ __device__ __forceinline__ void flux_march_item(const Dims& g, const PrimIn<T>& 
             const T ps = met_t<T>(psi[lin(g, cs[0], cs[1], cs[2])]), p2 = ps * ps;
             ip6 = rcp_t(p2 * p2 * p2);
         }
-        x[8] = (T)cell_qB_in(g, prim, bf, T1, cs, mi) * ip6;
-        x[9] = (T)cell_qB_in(g, prim, bf, T2, cs, mi) * ip6;
+        x[8] = prim.p[8 + T1][mi] * ip6;
+        x[9] = prim.p[8 + T2][mi] * ip6;
     };
     Rec rec[NV];
     {
-        T w[Rec::NINIT][NV];
+        T w[2][NV];
 #pragma unroll
-        for (int k = 0; k < Rec::NINIT; k++) load(f0 - Rec::NINIT + Rec::AHEAD + k, w[k]);
+        for (int k = 0; k < 2; k++) load(f0 - Rec::WARM + Rec::AHEAD - 2 + k, w[k]);
 #pragma unroll
         for (int v = 0; v < NV; v++) {
-            T x[Rec::NINIT];
-#pragma unroll
-            for (int k = 0; k < Rec::NINIT; k++) x[k] = w[k][v];
-            rec[v].init(x);
+            rec[v].push(w[0][v]);
+            rec[v].push(w[1][v]);
         }
     }
     int cm[3] = {c[0], c[1], c[2]};
     cm[D] = f0 - 1;
     long long rm = lin(g, cm[0], cm[1], cm[2]);
-    for (int f = f0; f < f1; f++) {
+    for (int f = f0 - Rec::WARM; f < f1; f++) {
         T x[NV];
         load(f + Rec::AHEAD, x);
-        T prL[8], prR[8], BL[3], BR[3];
-#pragma unroll
-        for (int v = 0; v < 8; v++) rec[v].step(x[v], prL[v], prR[v]);
-        rec[8].step(x[8], BL[T1], BR[T1]);
-        rec[9].step(x[9], BL[T2], BR[T2]);
+        T prL[NV], prR[NV];
+        line_step<NV>(rec, x, prL, prR);
+        if (f < f0) continue;
+        T BL[3], BR[3];
+        BL[T1] = prL[8];
+        BL[T2] = prL[9];
+        BR[T1] = prR[8];
+        BR[T2] = prR[9];
         c[D] = f;
         const long long r0 = lin(g, c[0], c[1], c[2]);
-        face_flux<D, M, T>(g, bf, psi_in, alp_in, c, rm, r0, prL, prR, BL, BR, F, vbar, Eh);
+        face_flux32<D, M>(g, bf, psi_in, alp_in, c, rm, r0, prL, prR, BL, BR, F, Eh);
         rm = r0;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// the FP64 face fluxes
+// ---------------------------------------------------------------------------
+
+// One side's half g = f + SG q of the unit-speed HLL flux in flat space, FP64, in the
+// frame (n, t1, t2) of the face (the quantities of face_hll_half, which lists them).  With
+//   e1 = B_t2 + SG E_t1,  e2 = SG E_t2 - B_t1   (the halves of E_t1 and E_t2)
+// the Maxwell terms of each momentum half collect, since SG^2 = 1:
+//   (E_t^2 + B_t^2) / 2 + SG (E x B)_n           = (e1^2 + e2^2) / 2
+//   -E_n E_t1 - B_n B_t1 + SG (E x B)_t1         = -SG E_n e1 + B_n e2
+//   -E_n E_t2 - B_n B_t2 + SG (E x B)_t2         = -SG E_n e2 - B_n e1
+// so that with a = u_n + SG W, N = (E_n^2 + B_n^2) / 2 and Q = (e1^2 + e2^2) / 2
+//   S_n: rho h a u_n + Q + (p - N),   tau: a (rho h W - rho) + SG (Q - (p - N)).
+// 30 FP64 instructions where the separate terms took 45.  W = s (1 + e/2 + 3 e^2 / 8) from
+// an FP32 estimate y of 1/sqrt(x): s = x y, e = 1 - s y (as in rsqrt_ge1).
+// st: rho, u_n, u_t1, u_t2, p, E_n, E_t1, E_t2; Bt: B_t1, B_t2; hBn2 = B_n^2 / 2.
+template <int SG>
+__device__ __forceinline__ void hll_half64(const double* st, const double* Bt, double Bn, double hBn2, double gh,
+                                           double* g, double& W)
+{
+    constexpr double sg = SG;
+    const double rho = st[0], u0 = st[1], u1 = st[2], u2 = st[3], p = st[4], En = st[5];
+    const double x = fma(u0, u0, fma(u1, u1, fma(u2, u2, 1.0)));
+    const double y = f2d_int(rsqrtf(d2f_int(x)));
+    const double s = x * y, e = fma(-s, y, 1.0);
+    W = fma(s, e * fma(0.375, e, 0.5), s);
+    const double h = fma(gh, p, rho), hW = h * W;
+    const double e1 = SG > 0 ? Bt[1] + st[6] : Bt[1] - st[6];
+    const double e2 = SG > 0 ? st[7] - Bt[0] : -st[7] - Bt[0];
+    const double Q2 = fma(e1, e1, e2 * e2);
+    const double pm = fma(-0.5 * En, En, p - hBn2);
+    const double a = SG > 0 ? u0 + W : u0 - W;
+    const double K = h * a;
+    g[0] = rho * a;
+    g[1] = fma(K, u0, fma(0.5, Q2, pm));
+    g[2] = fma(K, u1, fma(-sg * En, e1, Bn * e2));
+    g[3] = fma(K, u2, fma(-sg * En, e2, -Bn * e1));
+    g[4] = fma(a, hW - rho, SG > 0 ? fma(0.5, Q2, -pm) : fma(-0.5, Q2, pm));
+    g[5] = sg * En;
+    g[6] = e1;
+    g[7] = e2;
+}
+
+// Threads per block of the kernels that run flux64_item, and the shared doubles it takes
+// (SL per thread and quantity: MC a, b, lo, hi; PPM a0, a1, s0, ip, lo, hi)
+template <bool P, bool CC>
+struct Flux64 {
+    static constexpr int NV = CC ? 12 : 10;        // 8 primitives, B_t1, B_t2 (CC: B_n, B_t1, B_t2, Phi)
+    static constexpr int SL = P ? 6 : 4;
+    static constexpr int NT = !P ? 128 : (CC ? 64 : 96);
+    static constexpr int SM = NV * SL * NT;        // at most 48 KB
+};
+
+// The FP64 fluxes of K consecutive d-faces per thread, marched along d; CC: the 12
+// variables of the GLM scheme (cell-centred q_B in bq, q_Phi).
+//
+// A thread goes from cell to cell: it reconstructs the cell's two edge states, forms the
+// right state's half of the HLL flux at the lower face and completes that face, then the
+// left state's half at the upper face, which it carries to the next cell.  The cell
+// windows and edge states of the NV quantities lie in the thread's column of shared
+// memory, so that the reconstruction is a short rolled loop: held in registers it was
+// unrolled NV-fold, which took 168 registers (three blocks per SM) and a loop body beyond
+// the instruction cache (a fifth of the stalls were instruction fetches).  The direction
+// is a run-time value (the components are permuted as they are loaded), so that the tasks
+// of a launch share one code.
+//
+// Eh (flat metric, CT; NULL or with NULL entries): the edge EMFs along the directions
+// C != d whose third direction is inactive (1-D and 2-D grids).  Those edges coincide
+// with the d-faces, and uct_edge with the inactive side's two states equal and unit
+// speeds leaves (E_L + E_R -/+ the jump of the transverse q_B along d) / 2, which is half
+// the difference of the two HLL halves of E_C.
+template <bool M, bool P, bool CC>
+__device__ __forceinline__ void flux64_item(const Dims& g, int d, const double* const* prim, const double* const* bq,
+                                            const double* __restrict__ qphi, const double* psi_in,
+                                            const double* alp_in, double* const* F, double* const* vbar,
+                                            double* const* Eh, double* sm, long long t)
+{
+    using C = Flux64<P, CC>;
+    constexpr int NV = C::NV, SL = C::SL, NT = C::NT, G = CC ? 4 : 5;   // quantities in groups of G
+    constexpr int LO = SL - 2, HI = SL - 1;
+    constexpr int NF = CC ? 12 : 8;
+    const double* __restrict__ psi = M ? psi_in : nullptr;
+    const double* __restrict__ alp = M ? alp_in : nullptr;
+    double* const col = sm + threadIdx.x;
+    const int t1 = d == 2 ? 0 : d + 1, t2 = d == 0 ? 2 : d - 1;
+    // the line's chunk of faces f0 .. f1-1 and the offset of its cells at d-coordinate 0
+    int idx[3];
+    box_coords(t, d == 0 ? g.dq[0] : g.dv[0], d == 1 ? g.dq[1] : g.dv[1], idx);
+    const int q0 = d == 0 ? idx[0] : (d == 1 ? idx[1] : idx[2]);
+    const int f0 = g.ng[d] + q0 * g.mk[d], f1 = min(f0 + g.mk[d], g.ng[d] + g.n[d] + 1);
+    long long line = 0;
+    long long up[2] = {0, 0};   // from a cell's lower t1 / t2 face to its upper one
+#pragma unroll
+    for (int e = 0; e < 3; e++) {
+        if (e == d) continue;
+        const int ce = g.ng[e] + idx[e];
+        line += ce * g.st[e];
+        const int he = g.bc[e] == BC_PERIODIC && ce + 1 == g.ng[e] + g.n[e] ? g.ng[e] : ce + 1;
+        if (g.act[e]) up[e == t1 ? 0 : 1] = (he - ce) * g.st[e];
+    }
+    const long long sd = g.st[d];
+    // psi^2 and alpha at the face carried along, its normal B, and the left state's halves
+    double pf2 = 1.0, alf = 1.0, Bn = 0.0, hBn2 = 0.0, gL[NF], vL[2] = {0.0, 0.0};
+#pragma unroll
+    for (int v = 0; v < NF; v++) gL[v] = 0.0;
+    // one side's half flux at the carried face from the edge states in `slot`
+    auto half = [&](int slot, auto sgc, double* gh, double* vh) {
+        constexpr int SG = decltype(sgc)::value;
+        double pr[8], B[3], W;   // B: n, t1, t2
+#pragma unroll
+        for (int v = 0; v < 8; v++) pr[v] = col[(v * SL + slot) * NT];
+        if (CC) {
+#pragma unroll
+            for (int e = 0; e < 3; e++) B[e] = col[((8 + e) * SL + slot) * NT];
+        } else {
+            B[0] = Bn;
+            B[1] = col[(8 * SL + slot) * NT];
+            B[2] = col[(9 * SL + slot) * NT];
+        }
+        if (psi) {
+            // orthonormal frame: u_hat = psi^2 u, E_hat = psi^2 E, B_hat = psi^2 B
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                pr[1 + i] *= pf2;
+                pr[5 + i] *= pf2;
+                if (CC || i > 0) B[i] *= pf2;
+            }
+        }
+        if (CC) hBn2 = 0.5 * B[0] * B[0];
+        hll_half64<SG>(pr, B + 1, B[0], hBn2, g.gh, gh, W);
+        if (CC) {
+            // unit-speed halves of q_B (f_B^j = eta^{jnk} E_k) and of q_Phi (f = B^n)
+            gh[8] = SG * B[0];
+            gh[9] = SG * B[1] - pr[7];
+            gh[10] = SG * B[2] + pr[6];
+            gh[11] = B[0] + SG * col[(11 * SL + slot) * NT];
+        }
+        if (vbar && vbar[0]) {
+            const double iW = rcp_pos(W);
+            vh[0] = pr[2] * iW;
+            vh[1] = pr[3] * iW;
+        }
+    };
+    // centre cell m takes cell m + AHEAD; the first cells fill the windows
+    constexpr int AHEAD = P ? 2 : 1, WARM = P ? 2 : 0;
+    for (int m = f0 - 3 - WARM; m < f1; m++) {
+        const int mx = P ? ext_cell(g, d, m + AHEAD) : m + AHEAD;
+        const long long mi = chk(g, line + map_cell(g, d, mx) * sd);
+        double ip6 = 1.0;
+        if (psi) {
+            const double ps = psi[chk(g, line + mx * sd)], p2 = ps * ps;
+            ip6 = rcp_pos(p2 * p2 * p2);
+        }
+#pragma unroll 1
+        for (int q = 0; q < NV / G; q++) {
+            double x[G];
+            if (CC) {
+                if (q == 0) {
+                    x[0] = prim[0][mi];
+                    x[1] = prim[1 + d][mi];
+                    x[2] = prim[1 + t1][mi];
+                    x[3] = prim[1 + t2][mi];
+                } else if (q == 1) {
+                    x[0] = prim[4][mi];
+                    x[1] = prim[5 + d][mi];
+                    x[2] = prim[5 + t1][mi];
+                    x[3] = prim[5 + t2][mi];
+                } else {
+                    x[0] = bq[d][mi] * ip6;
+                    x[1] = bq[t1][mi] * ip6;
+                    x[2] = bq[t2][mi] * ip6;
+                    x[3] = qphi[mi] * ip6;
+                }
+            } else if (q == 0) {
+                x[0] = prim[0][mi];
+                x[1] = prim[1 + d][mi];
+                x[2] = prim[1 + t1][mi];
+                x[3] = prim[1 + t2][mi];
+                x[G - 1] = prim[4][mi];
+            } else {
+                x[0] = prim[5 + d][mi];
+                x[1] = prim[5 + t1][mi];
+                x[2] = prim[5 + t2][mi];
+                // the mean of the cell's two faces (an inactive direction: the cell value twice)
+                x[3] = scale_pow2<double, -1>(bq[t1][mi] + bq[t1][chk(g, mi + up[0])]) * ip6;
+                x[G - 1] = scale_pow2<double, -1>(bq[t2][mi] + bq[t2][chk(g, mi + up[1])]) * ip6;
+            }
+            double* const w = col + q * (G * SL * NT);
+            if (m < f0 - 1 - WARM) {
+#pragma unroll
+                for (int i = 0; i < G; i++) {
+                    double* const s = w + i * (SL * NT);
+                    s[0] = s[NT];
+                    s[NT] = x[i];
+                    if (P) {
+                        s[2 * NT] = 0.0;
+                        s[3 * NT] = x[i];
+                    }
+                }
+                continue;
+            }
+            unsigned redo = 0;
+#pragma unroll
+            for (int i = 0; i < G; i++) {
+                double* const s = w + i * (SL * NT);
+                double lo, hi;
+                if (P) {
+                    double in, s1;
+                    if (!fx_ppm_cell(s[0], s[NT], x[i], s[2 * NT], s[3 * NT], lo, hi, in, s1))
+                        ppm_cell<double>(s[0], s[NT], x[i], s[2 * NT], s[3 * NT], lo, hi, in, s1);
+                    s[0] = s[NT];
+                    s[NT] = x[i];
+                    s[2 * NT] = s1;
+                    s[3 * NT] = in;
+                } else {
+                    if (!fx_mc_cell(s[0], s[NT], x[i], lo, hi)) redo |= 1u << i;
+                }
+                s[LO * NT] = lo;
+                s[HI * NT] = hi;
+            }
+            if (!P) {
+                if (redo) {
+#pragma unroll 1
+                    for (int i = 0; i < G; i++) {
+                        double* const s = w + i * (SL * NT);
+                        double xi = x[0];
+#pragma unroll
+                        for (int j = 1; j < G; j++)
+                            if (i == j) xi = x[j];
+                        if (redo >> i & 1u) mc_cell_f64(s[0], s[NT], xi, s[LO * NT], s[HI * NT]);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < G; i++) {
+                    double* const s = w + i * (SL * NT);
+                    s[0] = s[NT];
+                    s[NT] = x[i];
+                }
+            }
+        }
+        if (m < f0 - 1) continue;
+        const long long r0 = chk(g, line + m * sd);
+        if (m >= f0) {
+            // HLL with c+ = c- = c = alpha sqrt(gamma^nn) = alpha / psi^2 (Sec. 2.5, maximal
+            // diffusivity): (c f_L + c f_R - c^2 (q_R - q_L)) / 2c = (f_L + f_R - c (q_R -
+            // q_L)) / 2.  Each densitised q_v is psi^k_v times its flat-space (psi = alpha = 1)
+            // value and its flux alpha psi^(k_v - 2) times, k = 6, 8, 8, 8, 6, 4, 4, 4 (GLM:
+            // and 4, 4, 4, 6): the HLL flux is then alpha psi^(k_v - 2) times the flat-space
+            // HLL flux (unit speed) of the orthonormal states.  F stores twice the flux (the
+            // update folds the 1/2).
+            double gR[NF], vR[2];
+            half(LO, SignConst<-1>(), gR, vR);
+            const double h2 = alf * pf2, h4 = h2 * pf2, h6 = h4 * pf2;
+            const int o[NF > 8 ? 12 : 8] = {0, 1 + d, 1 + t1, 1 + t2, 4, 5 + d, 5 + t1, 5 + t2};
+#pragma unroll
+            for (int v = 0; v < NF; v++) {
+                const double hv = v == 0 || v == 4 || v == 11 ? h4 : (v < 4 ? h6 : h2);
+                const int ov = v < 8 ? o[v < 8 ? v : 0] : (v == 8 ? 8 + d : (v == 9 ? 8 + t1 : (v == 10 ? 8 + t2 : 11)));
+                F[ov][r0] = (gL[v] + gR[v]) * hv;
+            }
+            if (!M && !CC && Eh) {
+                if (Eh[t1]) Eh[t1][r0] = scale_pow2<double, -1>(gL[6] - gR[6]);
+                if (Eh[t2]) Eh[t2][r0] = scale_pow2<double, -1>(gL[7] - gR[7]);
+            }
+            if (vbar && vbar[0]) {
+                // App. A steps (i)-(ii): vhat^j = alpha v^j (beta = 0) of the L and R states,
+                // vbar^j = (c- vhat^j_R + c+ vhat^j_L)/(c- + c+), their mean for c+ = c-;
+                // v^j = u_hat^j / (psi^2 W)
+                const double al = 0.5 * alf * (psi ? rcp_pos(pf2) : 1.0);
+                vbar[0][r0] = al * (vL[0] + vR[0]);
+                vbar[1][r0] = al * (vL[1] + vR[1]);
+            }
+        }
+        if (m + 1 < f1) {
+            const long long r1 = chk(g, r0 + sd);
+            const double psf = psi ? mean2<double>(psi[r0], psi[r1]) : 1.0;
+            alf = alp ? mean2<double>(alp[r0], alp[r1]) : 1.0;
+            pf2 = psf * psf;
+            if (!CC) {
+                Bn = bq[d][chk(g, line + map_face(g, d, m + 1) * sd)];   // B_hat: q_B / psi^4
+                if (psi) {
+                    const double i2 = rcp_pos(pf2);
+                    Bn *= i2 * i2;
+                }
+                hBn2 = 0.5 * Bn * Bn;
+            }
+            half(HI, SignConst<1>(), gL, vL);
+        }
     }
 }
 
@@ -587,24 +913,22 @@ __device__ __forceinline__ void emf_march_item(const Dims& g, const PrimIn<T>& p
         x[2] = (T)bf.p[A][face_at(g, A, cs)];
     };
     Rec rec[3];
-    {
-        T w[Rec::NINIT][3];
 #pragma unroll
-        for (int k = 0; k < Rec::NINIT; k++) row(f0 - Rec::NINIT + Rec::AHEAD + k, w[k]);
-#pragma unroll
-        for (int v = 0; v < 3; v++) {
-            T x[Rec::NINIT];
-#pragma unroll
-            for (int k = 0; k < Rec::NINIT; k++) x[k] = w[k][v];
-            rec[v].init(x);
-        }
+    for (int v = 0; v < 3; v++) {
+        rec[v].push(T(0));
+        rec[v].push(T(0));
     }
-    for (int f = f0; f < f1; f++) {
+    for (int f = f0 - Rec::WARM - 2; f < f1; f++) {
         T x3[3];
         row(f + Rec::AHEAD, x3);
-        T L[3], R[3];
+        if (f < f0 - Rec::WARM) {
 #pragma unroll
-        for (int v = 0; v < 3; v++) rec[v].step(x3[v], L[v], R[v]);
+            for (int v = 0; v < 3; v++) rec[v].push(x3[v]);
+            continue;
+        }
+        T L[3], R[3];
+        line_step<3>(rec, x3, L, R);
+        if (f < f0) continue;
         c[B] = f;
         // q_B^B (B-faces) along A
         T qBbL, qBbR;
@@ -636,6 +960,101 @@ __device__ __forceinline__ void emf_march_item(const Dims& g, const PrimIn<T>& p
         // lower-B state)
         Eh[i0] = to_f64(uct_edge<T>(ale * L[0], ale * R[0], ale * L[1], ale * R[1], ca, cb, qBbL, qBbR, L[2],
                                      R[2]));
+    }
+}
+
+// emf_march_item in FP64 with the edge direction C a run-time value (the launch's tasks
+// share one code) and the line's offsets formed once: the same reconstructions and sums.
+template <bool M, bool P>
+__device__ __forceinline__ void emf64_item(const Dims& g, int C, const double* const* prim, const double* const* bf,
+                                           const double* psi_in, const double* alp_in, double* __restrict__ Eh,
+                                           long long t)
+{
+    using Rec = LineRec<double, P>;
+    constexpr int NS = P ? 6 : 4, OFF = P ? 3 : 2;
+    const double* __restrict__ psi = M ? psi_in : nullptr;
+    const double* __restrict__ alp = M ? alp_in : nullptr;
+    const int A = C == 2 ? 0 : C + 1, B = C == 0 ? 2 : C - 1;
+    const double* __restrict__ Ec = prim[5 + C];
+    const double* __restrict__ qA = bf[A];
+    const double* __restrict__ qB = bf[B];
+    // x-fastest box: the chunks along B, n[C] edges along C, n[A] + 1 along A
+    int idx[3];
+    box_coords(t, B == 0 ? g.dq[0] : (C == 0 ? g.dv[0] : g.dvp[0]), B == 1 ? g.dq[1] : (C == 1 ? g.dv[1] : g.dvp[1]),
+               idx);
+    auto at = [&](int d) { return d == 0 ? idx[0] : (d == 1 ? idx[1] : idx[2]); };
+    const int f0 = g.ng[B] + at(B) * g.mk[B], f1 = min(f0 + g.mk[B], g.ng[B] + g.n[B] + 1);
+    const int cA = g.ng[A] + at(A);
+    const long long line = (g.ng[C] + at(C)) * g.st[C], sA = g.st[A], sB = g.st[B];
+    // the cells along A around the edge (mapped, and where the metric is read), its A-face
+    long long ia[NS], pa[NS];
+#pragma unroll
+    for (int k = 0; k < NS; k++) {
+        const int m = P ? ext_cell(g, A, cA + k - OFF) : cA + k - OFF;
+        ia[k] = line + map_cell(g, A, m) * sA;
+        pa[k] = line + m * sA;
+    }
+    const long long fa = line + map_face(g, A, cA) * sA;
+    auto recA = [&](const double* v, double& L, double& R) {
+        if (P) ppm_face<double>(v, L, R);
+        else mc_face<double>(v[0], v[1], v[2], v[NS - 1], L, R);
+    };
+    Rec rec[3];
+#pragma unroll
+    for (int v = 0; v < 3; v++) {
+        rec[v].push(0.0);
+        rec[v].push(0.0);
+    }
+    for (int f = f0 - Rec::WARM - 2; f < f1; f++) {
+        // row f + AHEAD along B: covariant E_C = psi^4 E^C reconstructed along A to the
+        // A-face, and q_B^A at that A-face
+        const int mb = P ? ext_cell(g, B, f + Rec::AHEAD) : f + Rec::AHEAD;
+        const long long rb = map_cell(g, B, mb) * sB;
+        double x3[3];
+        {
+            double v[NS];
+#pragma unroll
+            for (int k = 0; k < NS; k++) {
+                v[k] = Ec[chk(g, ia[k] + rb)];
+                if (psi) {
+                    const double ps = psi[chk(g, pa[k] + mb * sB)], p2 = ps * ps;
+                    v[k] *= p2 * p2;
+                }
+            }
+            recA(v, x3[0], x3[1]);
+        }
+        x3[2] = qA[chk(g, fa + rb)];
+        if (f < f0 - Rec::WARM) {
+#pragma unroll
+            for (int v = 0; v < 3; v++) rec[v].push(x3[v]);
+            continue;
+        }
+        double L[3], R[3];
+        line_step<3>(rec, x3, L, R);
+        if (f < f0) continue;
+        // q_B^B (B-faces) along A
+        double qL, qR;
+        {
+            const long long jb = map_face(g, B, f) * sB;
+            double v[NS];
+#pragma unroll
+            for (int k = 0; k < NS; k++) v[k] = qB[chk(g, ia[k] + jb)];
+            recA(v, qL, qR);
+        }
+        const long long i0 = chk(g, line + cA * sA + f * sB);
+        double ale = 1.0, ca = 1.0, cb = 1.0;
+        if (alp || psi) {
+            double sum = alp ? alp[i0] : 1.0;
+            sum += alp ? alp[chk(g, i0 - sA)] : 1.0;
+            sum += alp ? alp[chk(g, i0 - sB)] : 1.0;
+            sum += alp ? alp[chk(g, i0 - sA - sB)] : 1.0;
+            ale = sum * 0.25;
+            double cab[2];
+            edge_speeds<double>(g, psi, alp, i0, true, true, sA, sB, cab);
+            ca = cab[0];
+            cb = cab[1];
+        }
+        Eh[i0] = uct_edge<double>(ale * L[0], ale * R[0], ale * L[1], ale * R[1], ca, cb, qL, qR, L[2], R[2]);
     }
 }
 

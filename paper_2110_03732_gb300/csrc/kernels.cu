@@ -1,9 +1,10 @@
 // CUDA kernels of one IMEX-RK stage of resistive (GR)MHD with staggered
 // constrained transport (arXiv 2110.03732), sm_103a, FP64 and mixed precision.
 //
-//   k_implicit   Sec. 2.4: per-cell Newton on u coupled to the implicit E update;
+// In this file: the update, the set-up kernels and the reductions.  The others:
+//   k_implicit (implicit.cu)  Sec. 2.4: per-cell Newton on u coupled to the implicit E update;
 //                writes stage primitives and the stiff rate R = (q_E - q_E,base)/(a_ii dt)
-//   k_stencil<M, T, P>  one launch per stage of
+//   k_stencil<M, T, P> (stencil.cuh)  one launch per stage of
 //                - the flux tasks, Sec. 2.1 + Sec. 5 defaults: MC (or PPM)
 //                  reconstruction to the D-faces, marched along D, and the HLL flux with
 //                  the maximal-diffusivity speeds of Sec. 2.5 (on flat 1-D / 2-D grids
@@ -12,7 +13,7 @@
 //                  edge EMF hat{E}_C, marched along C + 2 when both transverse
 //                  directions are active
 //                in FP64 or (T = float) mixed precision
-//   k_flux_march<D>, k_emf_ideal<C>  the fluxes and App. A edge EMF of the ideal-limit
+//   k_flux_march<D>, k_emf_ideal<C> (flux.cu)  the fluxes and App. A edge EMF of the ideal-limit
 //                variant (separate launches: the flux writes the transport velocities)
 //   k_update<M>  flux divergence + non-stiff sources (Sec. 2.1) and the CT face update
 //                (Sec. 3.2); writes L, or folds it straight into the IMEX stage bases and
@@ -20,157 +21,15 @@
 //   k_prim2con, k_curlA (Sec. 4), k_dt (Sec. 2.5), k_divb, k_totals: set-up and
 //   diagnostics; k_implicit_cc, k_curlA_cc, k_prim2con_cc, k_diag_cc: the same for the
 //   cell-centred fields of the GLM variant (its flux and update kernels: glm.cu)
-#include <cstring>
-
 #include "grmhd_device.cuh"
 #include "items.cuh"
 #include "kernels.h"
 #include "launch.cuh"
+#include "stencil.cuh"
 
 namespace grmhd {
 
 thread_local bool launch_overlap = false;
-
-// ---------------------------------------------------------------------------
-// implicit step
-// ---------------------------------------------------------------------------
-
-// Five blocks per SM (96 registers, about 1 KB of spills): against four (128 registers)
-// the mixed-precision and metric instances ran 1.5-4 % faster (512^2 vortex mixed 58.1 ->
-// 57.3 us, 128^3 star mixed 398 -> 381 us, FP64 455 -> 442 us per launch); the flat FP64
-// instance is unchanged (79.3 us).
-template <bool M, bool ACC>
-__global__ void __launch_bounds__(128, 5) k_implicit(Dims g, ImpArgs a)
-{
-    grid_dep_sync();
-    const long long tot = (long long)g.n[0] * g.n[1] * g.n[2];
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot;
-         t += (long long)gridDim.x * blockDim.x)
-        implicit_item<M, false, ACC>(g, a, t);
-}
-
-// the same solve with cell-centred q_B (GLM variant, Sec. 3.1)
-template <bool M>
-__global__ void __launch_bounds__(128, 4) k_implicit_cc(Dims g, ImpArgs a)
-{
-    grid_dep_sync();
-    const long long tot = (long long)g.n[0] * g.n[1] * g.n[2];
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot;
-         t += (long long)gridDim.x * blockDim.x)
-        implicit_item<M, true>(g, a, t);
-}
-
-// ---------------------------------------------------------------------------
-// face fluxes
-// ---------------------------------------------------------------------------
-
-// MC (or PPM) fluxes, K consecutive D-faces per thread (flux_march_item)
-template <int D, bool M, typename T, bool P = false>
-__global__ void __launch_bounds__(128) k_flux_march(Dims g, FluxArgs<T> a)
-{
-    grid_dep_sync();
-    const long long nq = g.dq[D].d;   // chunks of g.mk[D] faces per line
-    const long long tot = nq * (D == 0 ? (long long)g.n[1] * g.n[2]
-                                       : (D == 1 ? (long long)g.n[0] * g.n[2] : (long long)g.n[0] * g.n[1]));
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot;
-         t += (long long)gridDim.x * blockDim.x)
-        flux_march_item<D, M, T, P>(g, a.prim, a.bf, a.psi, a.alp, a.F, a.vbar, a.Eh, t);
-}
-
-// ---------------------------------------------------------------------------
-// the explicit stencil of a stage: face fluxes and upwind constrained transport
-// (hat{E}_C on the edges along C, stored at the corner index that is lower in
-// a = C+1 and b = C+2)
-// ---------------------------------------------------------------------------
-
-// The face fluxes of every active direction and the edge EMFs the flux tasks do not
-// write, in one launch (resistive UCT, FP64 or mixed precision).  Block ranges select
-// the task (the same items, march lengths and grid copies as separate launches would
-// take, so every face and edge is bitwise the same); one launch keeps the SMs filled
-// across what would be three to six single-wave kernels with their tails.
-template <typename T>
-struct StencilTasks {
-    int b0[7];                 // first block of task s (flux x, y, z; EMF x, y, z); b0[6] = grid
-    int emarch[3];             // EMF task C marches along C + 2 (both transverse directions active)
-    Dims g[6];                 // each task's copy of the grid, with its march length
-    FluxArgs<T> fa[3];
-    EmfArgs<T> ea[3];
-};
-
-template <int D, bool M, typename T, bool P>
-__device__ __forceinline__ void stencil_flux(const Dims& g, const FluxArgs<T>& a, long long t0, long long nt)
-{
-    const long long tot = g.dq[D].d * (D == 0 ? (long long)g.n[1] * g.n[2]
-                                              : (D == 1 ? (long long)g.n[0] * g.n[2] : (long long)g.n[0] * g.n[1]));
-    for (long long t = t0; t < tot; t += nt)
-        flux_march_item<D, M, T, P>(g, a.prim, a.bf, a.psi, a.alp, a.F, nullptr, a.Eh, t);
-}
-
-template <int C, bool M, typename T, bool P>
-__device__ __forceinline__ void stencil_emf(const Dims& g, const EmfArgs<T>& a, int march, long long t0,
-                                            long long nt)
-{
-    constexpr int A = (C + 1) % 3, B = (C + 2) % 3;
-    if (march) {
-        const long long tot = (long long)g.dq[B].d * g.n[C] * (g.n[A] + 1);
-        for (long long t = t0; t < tot; t += nt) emf_march_item<C, M, T, P>(g, a.prim, a.bf, a.psi, a.alp, a.Eh, t);
-    } else {
-        long long tot = 1;
-#pragma unroll
-        for (int d = 0; d < 3; d++) tot *= (d == C) ? g.n[d] : (g.act[d] ? g.n[d] + 1 : 1);
-        for (long long t = t0; t < tot; t += nt) emf_item<C, M, T, P>(g, a.prim, a.bf, a.psi, a.alp, a.Eh, t);
-    }
-}
-
-// The FP32 PPM instance is held to 96 registers (five blocks per SM, 160 B of spills):
-// at its natural 128 it ran 2 % slower.  The others keep the compiler's choice.
-template <bool M, typename T, bool P>
-__global__ void __launch_bounds__(128, (sizeof(T) == 4 && P) ? 5 : 0) k_stencil(StencilTasks<T> L)
-{
-    grid_dep_sync();
-    const int b = blockIdx.x;
-    int s = 0;
-#pragma unroll
-    for (int i = 1; i < 6; i++)
-        if (b >= L.b0[i]) s = i;   // empty tasks have b0[i] == b0[i + 1]
-    switch (s) {
-#define GRMHD_STENCIL_CASE(S, CALL)                                                   \
-    case S: {                                                                         \
-        const long long nt = (long long)(L.b0[S + 1] - L.b0[S]) * blockDim.x;        \
-        const long long t0 = (long long)(b - L.b0[S]) * blockDim.x + threadIdx.x;    \
-        CALL;                                                                         \
-        break;                                                                        \
-    }
-        GRMHD_STENCIL_CASE(0, (stencil_flux<0, M, T, P>(L.g[0], L.fa[0], t0, nt)))
-        GRMHD_STENCIL_CASE(1, (stencil_flux<1, M, T, P>(L.g[1], L.fa[1], t0, nt)))
-        GRMHD_STENCIL_CASE(2, (stencil_flux<2, M, T, P>(L.g[2], L.fa[2], t0, nt)))
-        GRMHD_STENCIL_CASE(3, (stencil_emf<0, M, T, P>(L.g[3], L.ea[0], L.emarch[0], t0, nt)))
-        GRMHD_STENCIL_CASE(4, (stencil_emf<1, M, T, P>(L.g[4], L.ea[1], L.emarch[1], t0, nt)))
-        GRMHD_STENCIL_CASE(5, (stencil_emf<2, M, T, P>(L.g[5], L.ea[2], L.emarch[2], t0, nt)))
-#undef GRMHD_STENCIL_CASE
-    default: break;
-    }
-}
-
-// ideal-limit edge EMF (App. A) from the stored transport velocities
-struct VbarArgs {
-    const double* p[3][2];
-};
-
-template <int C, bool M>
-__global__ void __launch_bounds__(128) k_emf_ideal(Dims g, EmfArgs<double> a, VbarArgs vb)
-{
-    grid_dep_sync();
-    long long tot = 1;
-#pragma unroll
-    for (int d = 0; d < 3; d++) tot *= (d == C) ? g.n[d] : (g.act[d] ? g.n[d] + 1 : 1);
-    CP8 prim;
-#pragma unroll
-    for (int v = 0; v < 8; v++) prim.p[v] = a.prim.p[v];
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot;
-         t += (long long)gridDim.x * blockDim.x)
-        emf_ideal_item<C, M>(g, prim, a.bf, a.psi, a.alp, vb.p, a.Eh, t);
-}
 
 // ---------------------------------------------------------------------------
 // update: cell-centred L (flux divergence + non-stiff sources) and face L_B (CT)
@@ -448,24 +307,6 @@ __global__ void __launch_bounds__(256) k_fold(const double* __restrict__ part, i
 // launchers
 // ---------------------------------------------------------------------------
 
-static int grid_for(long long work, int threads, int nsm)
-{
-    long long b = (work + threads - 1) / threads;
-    const long long cap = (long long)nsm * 16;
-    if (b > cap) b = cap;
-    if (b < 1) b = 1;
-    return (int)b;
-}
-
-cudaError_t launch_implicit(const Dims& g, const ImpArgs& a, int nsm, cudaStream_t st)
-{
-    const long long work = (long long)g.n[0] * g.n[1] * g.n[2];
-    const bool m = a.psi || a.alp;
-    if (a.dwacc) launch_k(m ? k_implicit<true, true> : k_implicit<false, true>, grid_for(work, 128, nsm), 128, st, g, a);
-    else launch_k(m ? k_implicit<true, false> : k_implicit<false, false>, grid_for(work, 128, nsm), 128, st, g, a);
-    return cudaGetLastError();
-}
-
 __global__ void __launch_bounds__(256) k_hist_init(long long n, const double* __restrict__ u1,
                                                    const double* __restrict__ u2, const double* __restrict__ u3,
                                                    const double* __restrict__ psi, P3f hs, P3f hd)
@@ -486,159 +327,24 @@ cudaError_t launch_hist_init(const Dims& g, const double* u1, const double* u2, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_implicit_cc(const Dims& g, const ImpArgs& a, int nsm, cudaStream_t st)
-{
-    const long long work = (long long)g.n[0] * g.n[1] * g.n[2];
-    // GLM contexts are FP64 only: the FP64 residual accepts the root
-    launch_k(a.psi || a.alp ? k_implicit_cc<true> : k_implicit_cc<false>, grid_for(work, 128, nsm), 128, st, g,
-             a);
-    return cudaGetLastError();
-}
-
-
-// resident 128-thread blocks per SM of a marching flux kernel (its register count
-// decides: about 2 for FP64, 4 for FP32), queried once
-template <int D, bool M, typename T, bool P>
-static int march_blocks_per_sm()
-{
-    static int nb = 0;
-    if (nb < 1) {
-        int q = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_flux_march<D, M, T, P>, 128, 0) != cudaSuccess ||
-            q < 1)
-            q = 1;
-        nb = q;
-    }
-    return nb;
-}
-
-// faces per thread by march_len (start-up: 3 cells for MC, 5 for PPM, each about a
-// fifth of a face's work).  For FP64, waves are counted at no more than two resident
-// blocks per SM.  At 8 warps the FP64 flux already keeps the FP64 pipe ~75-80 % busy, and
-// a third block (where the registers allow it) adds no throughput.  A shorter march to
-// fill that block would only add start-ups: 5 faces at three blocks per SM took 123 us
-// per 512^2 launch, against 117 us for 7 faces at two.
-template <int D, bool M, typename T, bool P>
-static void flux_march_launch(const Dims& g, int nsm, cudaStream_t st, const FluxArgs<T>& a)
-{
-    const long long other = D == 0 ? (long long)g.n[1] * g.n[2]
-                                   : (D == 1 ? (long long)g.n[0] * g.n[2] : (long long)g.n[0] * g.n[1]);
-    const int bps = march_blocks_per_sm<D, M, T, P>();
-    const int K = march_len(g.n[D], other, nsm, sizeof(T) == 8 && bps > 2 ? 2 : bps, P ? 1.0 : 0.6);
-    Dims gl = g;
-    set_march(gl, D, K);
-    const int b = grid_for((long long)gl.dq[D].d * other, 128, nsm);
-    launch_k(k_flux_march<D, M, T, P>, b, 128, st, gl, a);
-}
-
-template <typename T, bool P>
-static void flux_dispatch(const Dims& g, int d, bool m, int nsm, cudaStream_t st, const FluxArgs<T>& a)
-{
-    if (d == 0) m ? flux_march_launch<0, true, T, P>(g, nsm, st, a) : flux_march_launch<0, false, T, P>(g, nsm, st, a);
-    else if (d == 1) m ? flux_march_launch<1, true, T, P>(g, nsm, st, a) : flux_march_launch<1, false, T, P>(g, nsm, st, a);
-    else m ? flux_march_launch<2, true, T, P>(g, nsm, st, a) : flux_march_launch<2, false, T, P>(g, nsm, st, a);
-}
-
-// edges of direction C (one per thread when A or B is inactive)
-static long long emf_work(const Dims& g, int c)
-{
-    long long work = 1;
-    for (int d = 0; d < 3; d++) work *= (d == c) ? g.n[d] : (g.act[d] ? g.n[d] + 1 : 1);
-    return work;
-}
-
-cudaError_t launch_flux(const Dims& g, int d, CP8 prim, CP3 bf, const double* psi, const double* alp, P8 F, int nsm,
-                        cudaStream_t st, double* const* vbar, bool ppm, double* const* Eh)
-{
-    FluxArgs<double> a;
-    for (int k = 0; k < 3; k++) a.Eh[k] = Eh && !(psi || alp) ? Eh[k] : nullptr;
-    for (int v = 0; v < 8; v++) {
-        a.prim.p[v] = prim.p[v];
-        a.F.p[v] = F.p[v];
-    }
-    a.vbar[0] = vbar ? vbar[0] : nullptr;
-    a.vbar[1] = vbar ? vbar[1] : nullptr;
-    a.bf = bf;
-    a.psi = psi;
-    a.alp = alp;
-    if (ppm) flux_dispatch<double, true>(g, d, psi || alp, nsm, st, a);
-    else flux_dispatch<double, false>(g, d, psi || alp, nsm, st, a);
-    return cudaGetLastError();
-}
-
-template <bool M, typename T, bool P>
-static int stencil_blocks_per_sm()
-{
-    static int nb = 0;
-    if (nb < 1) {
-        int q = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_stencil<M, T, P>, 128, 0) != cudaSuccess || q < 1)
-            q = 1;
-        nb = q;
-    }
-    return nb;
-}
-
 template <typename T>
-static cudaError_t stencil_launch(const Dims& g, const PrimIn<T>& prim, CP3 bf, const double* psi, const double* alp,
-                                  const FluxOut<T>* F, double* const (*fe)[3], double* const* Eh, int nsm,
-                                  cudaStream_t st, bool ppm)
+static cudaError_t stencil_dispatch(const Dims& g, const PrimIn<T>& prim, CP3 bf, const double* psi, const double* alp,
+                                    const FluxOut<T>* F, double* const (*fe)[3], double* const* Eh, int nsm,
+                                    cudaStream_t st, bool ppm)
 {
     const bool m = psi || alp;
-    const int bps = ppm ? (m ? stencil_blocks_per_sm<true, T, true>() : stencil_blocks_per_sm<false, T, true>())
-                        : (m ? stencil_blocks_per_sm<true, T, false>() : stencil_blocks_per_sm<false, T, false>());
-    const double c0 = ppm ? 1.0 : 0.6;
-    StencilTasks<T> L;
-    memset(&L, 0, sizeof L);
-    int nb = 0;
-    for (int d = 0; d < 3; d++) {
-        L.b0[d] = nb;
-        L.g[d] = g;
-        FluxArgs<T>& a = L.fa[d];
-        a.prim = prim;
-        a.bf = bf;
-        a.psi = psi;
-        a.alp = alp;
-        if (!g.act[d]) continue;
-        a.F = F[d];
-        for (int k = 0; k < 3; k++) a.Eh[k] = fe && !m ? fe[d][k] : nullptr;
-        const long long other = d == 0 ? (long long)g.n[1] * g.n[2]
-                                       : (d == 1 ? (long long)g.n[0] * g.n[2] : (long long)g.n[0] * g.n[1]);
-        set_march(L.g[d], d, march_len(g.n[d], other, nsm, bps, c0));
-        nb += grid_for((long long)L.g[d].dq[d].d * other, 128, nsm);
-    }
-    for (int c = 0; c < 3; c++) {
-        L.b0[3 + c] = nb;
-        L.g[3 + c] = g;
-        EmfArgs<T>& a = L.ea[c];
-        a.prim = prim;
-        a.bf = bf;
-        a.psi = psi;
-        a.alp = alp;
-        if (!Eh || !Eh[c]) continue;
-        a.Eh = Eh[c];
-        const int A = (c + 1) % 3, B = (c + 2) % 3;
-        if (g.act[A] && g.act[B]) {
-            const long long other = (long long)g.n[c] * (g.n[A] + 1);
-            set_march(L.g[3 + c], B, march_len(g.n[B], other, nsm, bps, c0));
-            L.emarch[c] = 1;
-            nb += grid_for((long long)L.g[3 + c].dq[B].d * other, 128, nsm);
-        } else {
-            nb += grid_for(emf_work(g, c), 128, nsm);
-        }
-    }
-    L.b0[6] = nb;
-    if (nb == 0) return cudaSuccess;
-    if (ppm) launch_k(m ? k_stencil<true, T, true> : k_stencil<false, T, true>, nb, 128, st, L);
-    else launch_k(m ? k_stencil<true, T, false> : k_stencil<false, T, false>, nb, 128, st, L);
-    return cudaGetLastError();
+    if (ppm)
+        return m ? stencil_launch<true, T, true>(g, prim, bf, psi, alp, F, fe, Eh, nsm, st)
+                 : stencil_launch<false, T, true>(g, prim, bf, psi, alp, F, fe, Eh, nsm, st);
+    return m ? stencil_launch<true, T, false>(g, prim, bf, psi, alp, F, fe, Eh, nsm, st)
+             : stencil_launch<false, T, false>(g, prim, bf, psi, alp, F, fe, Eh, nsm, st);
 }
 
 cudaError_t launch_stencil32(const Dims& g, const PrimIn<float>& prim, CP3 bf, const double* psi, const double* alp,
                              const FluxOut<float>* F, double* const (*fe)[3], double* const* Eh, int nsm,
                              cudaStream_t st, bool ppm)
 {
-    return stencil_launch<float>(g, prim, bf, psi, alp, F, fe, Eh, nsm, st, ppm);
+    return stencil_dispatch<float>(g, prim, bf, psi, alp, F, fe, Eh, nsm, st, ppm);
 }
 
 cudaError_t launch_stencil64(const Dims& g, CP8 prim, CP3 bf, const double* psi, const double* alp, const P8* F,
@@ -649,27 +355,7 @@ cudaError_t launch_stencil64(const Dims& g, CP8 prim, CP3 bf, const double* psi,
     for (int v = 0; v < 8; v++) p.p[v] = prim.p[v];
     for (int d = 0; d < 3; d++)
         for (int v = 0; v < 8; v++) fo[d].p[v] = F[d].p[v];
-    return stencil_launch<double>(g, p, bf, psi, alp, fo, fe, Eh, nsm, st, ppm);
-}
-
-cudaError_t launch_emf_ideal(const Dims& g, int c, CP8 prim, CP3 bf, const double* psi, const double* alp,
-                             const double* const (*vb)[2], double* Eh, int nsm, cudaStream_t st)
-{
-    EmfArgs<double> a;
-    for (int v = 0; v < 8; v++) a.prim.p[v] = prim.p[v];
-    a.bf = bf;
-    a.psi = psi;
-    a.alp = alp;
-    a.Eh = Eh;
-    VbarArgs v;
-    for (int d = 0; d < 3; d++)
-        for (int k = 0; k < 2; k++) v.p[d][k] = vb[d][k];
-    const int b = grid_for(emf_work(g, c), 128, nsm);
-    const bool m = psi || alp;
-    if (c == 0) launch_k(m ? k_emf_ideal<0, true> : k_emf_ideal<0, false>, b, 128, st, g, a, v);
-    else if (c == 1) launch_k(m ? k_emf_ideal<1, true> : k_emf_ideal<1, false>, b, 128, st, g, a, v);
-    else launch_k(m ? k_emf_ideal<2, true> : k_emf_ideal<2, false>, b, 128, st, g, a, v);
-    return cudaGetLastError();
+    return stencil_dispatch<double>(g, p, bf, psi, alp, fo, fe, Eh, nsm, st, ppm);
 }
 
 cudaError_t launch_update(const Dims& g, const UpdateArgs& a, int nsm, cudaStream_t st)

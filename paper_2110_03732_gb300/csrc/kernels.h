@@ -175,6 +175,13 @@ cudaError_t launch_diag_cc(const Dims& g, CP3 qB, CP8 q, double dV, double* part
 // index-bounds violations counted by each translation unit's kernels in a checked
 // build (GRMHD_CHECK_BOUNDS; 0 otherwise, ~0 if the counter could not be read)
 unsigned long long oob_kernels(bool reset);
+unsigned long long oob_implicit(bool reset);
+unsigned long long oob_flux(bool reset);
+unsigned long long oob_stencil64(bool reset);
+unsigned long long oob_stencil64m(bool reset);
+unsigned long long oob_stencil64p(bool reset);
+unsigned long long oob_stencil64mp(bool reset);
+unsigned long long oob_stencil32(bool reset);
 unsigned long long oob_glm(bool reset);
 unsigned long long oob_elliptic(bool reset);
 unsigned long long oob_batch(bool reset);
