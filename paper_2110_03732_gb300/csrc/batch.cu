@@ -74,8 +74,9 @@ constexpr int kMinItems = 128;   // smallest chunk of any candidate (scratch siz
 // batched kernels
 // ---------------------------------------------------------------------------
 
+// (64 registers, as k_implicit)
 template <bool M, bool ACC>
-__global__ void __launch_bounds__(256) kb_implicit(const ProbStage* __restrict__ P, int s, int stage,
+__global__ void __launch_bounds__(256, 4) kb_implicit(const ProbStage* __restrict__ P, int s, int stage,
                                                   const Chunk* __restrict__ ch, int nch)
 {
     for (int i = blockIdx.x; i < nch; i += gridDim.x) {

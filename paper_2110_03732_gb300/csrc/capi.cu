@@ -271,6 +271,7 @@ ImpArgs imp_args(grmhd_ctx* c, CP8 qb, CP3 bf, double a_dt, P8 prim, P3 R, P3 qE
     a.a_dt = a_dt;
     a.ia_dt = a_dt > 0.0 ? 1.0 / a_dt : 0.0;
     a.ighf = (float)c->g.igh;
+    a.ighl = (float)(c->g.igh - (double)a.ighf);
     a.xif = (float)c->xi;
     a.prim = prim;
     a.R = R;

@@ -85,6 +85,27 @@ __device__ __forceinline__ dw dw_sqr(dw x)
     return fast_two_sum(p, e);
 }
 
+// A product left as the rounded hi and all of its error in lo (|lo| up to about two last
+// places of hi): enough for a sum, which renormalises.
+__device__ __forceinline__ dw dw_mul_raw(dw x, dw y)
+{
+    const float p = __fmul_rn(x.hi, y.hi);
+    float e = fmaf(x.hi, y.hi, -p);
+    e = fmaf(x.hi, y.lo, e);
+    e = fmaf(x.lo, y.hi, e);
+    return {p, e};
+}
+
+// x + y with the errors gathered in lo, not renormalised (each further term of a sum adds
+// its error there; dw_norm at its end)
+__device__ __forceinline__ dw dw_add_raw(dw x, dw y)
+{
+    const dw s = two_sum(x.hi, y.hi);
+    return {s.hi, __fadd_rn(s.lo, __fadd_rn(x.lo, y.lo))};
+}
+
+__device__ __forceinline__ dw dw_norm(dw x) { return fast_two_sum(x.hi, x.lo); }
+
 // x * 2^k for a power-of-two factor s (exact unless it leaves the normal range)
 __device__ __forceinline__ dw dw_scale(dw x, float s) { return {__fmul_rn(x.hi, s), __fmul_rn(x.lo, s)}; }
 

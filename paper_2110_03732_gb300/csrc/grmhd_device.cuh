@@ -252,6 +252,16 @@ __device__ __forceinline__ double cell_qB(const Dims& g, const double* __restric
     return scale_pow2<double, -1>(bf[i0] + bf[i1]);
 }
 
+// the same for an interior cell c of linear index i0 (no mapping but the upper face's)
+__device__ __forceinline__ double cell_qB_in(const Dims& g, const double* __restrict__ bf, int e, const int* c,
+                                             long long i0)
+{
+    if (!g.act[e]) return bf[i0];
+    const bool wrap = g.bc[e] == BC_PERIODIC && c[e] + 1 == g.ng[e] + g.n[e];
+    const long long i1 = chk(g, i0 + (wrap ? 1 - g.n[e] : 1) * g.st[e]);
+    return scale_pow2<double, -1>(bf[i0] + bf[i1]);
+}
+
 // ---------------------------------------------------------------------------
 // MC limiter (monotonised central, van Leer 1974)
 //
@@ -822,6 +832,47 @@ __device__ __forceinline__ void evaluate(const CellIn& c, const double* u, Eval&
                       max(max(mag_hi(x1), mag_hi(x2)), max(mag_hi(w0), max(mag_hi(w1), mag_hi(w2))))));
 }
 
+// The residual at u in FP64 for the test that accepts a double-word root (emode 0 and 1):
+// evaluate()'s quantities with their sums as chains of fused multiply-adds and without the
+// momentum scale, which the caller has from the double-word evaluation before it.
+struct Accept {
+    double W, iW, wt, E[3], f[3];
+};
+
+__device__ __forceinline__ void evaluate_accept(const double D, const double tau, const double* S, const double* Es,
+                                                const double* B, double et, double igh, int emode, const double* u,
+                                                Accept& e)
+{
+    const double Wsq = fma(u[0], u[0], fma(u[1], u[1], fma(u[2], u[2], 1.0)));
+    e.iW = rsqrt_ge1(Wsq);
+    e.W = Wsq * e.iW;
+    const double d = Wsq - igh;
+    double iden;
+    if (emode == 1) {
+        // one reciprocal for 1/(W + eta_t), 1/(1 + eta_t W) and 1/(W^2 - 1/Gamma_hat)
+        const double a = e.W + et, b = fma(et, e.W, 1.0), ab = a * b, r = rcp_pos(ab * d), rd = r * d;
+        const double iWe = rd * b;
+        iden = r * ab;
+        const double ae = (et * (rd * a)) * fma(Es[0], u[0], fma(Es[1], u[1], Es[2] * u[2]));
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            const int j = (i + 1) % 3, k = (i + 2) % 3;
+            e.E[i] = fma(u[k], B[j], fma(-u[j], B[k], fma(ae, u[i], et * Es[i]))) * iWe;
+        }
+    } else {
+        iden = rcp_pos(d);
+#pragma unroll
+        for (int i = 0; i < 3; i++) e.E[i] = Es[i];
+    }
+    const double U2 = fma(B[0], B[0], fma(B[1], B[1], fma(B[2], B[2], fma(e.E[0], e.E[0], fma(e.E[1], e.E[1], e.E[2] * e.E[2])))));
+    e.wt = fma(e.W, fma(-0.5, U2, tau + D), -(D * igh)) * iden;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        const int j = (i + 1) % 3, k = (i + 2) % 3;
+        e.f[i] = fma(e.wt, u[i], fma(e.E[j], B[k], fma(-e.E[k], B[j], -S[i])));
+    }
+}
+
 // |f|^2 of an evaluated residual
 __device__ __forceinline__ double fnorm2(const Eval& e) { return e.f[0] * e.f[0] + e.f[1] * e.f[1] + e.f[2] * e.f[2]; }
 
@@ -917,10 +968,10 @@ __device__ __forceinline__ CellF cell_f32(const CellIn& c)
 }
 
 // E(u) and dE_i/du_j in FP32 at the FP32 velocity uf (W = Wf, 1/W = iWf)
-__device__ __forceinline__ void efield_f32(const CellIn& c, const CellF& cf, const float* uf, float Wf, float iWf,
+__device__ __forceinline__ void efield_f32(int emode, const CellF& cf, const float* uf, float Wf, float iWf,
                                            float* Ef, float dE[3][3])
 {
-    if (c.emode == 2) {
+    if (emode == 2) {
         DynT<float> dy;
         dyn_coeffs<float>(Wf, cf.etat, cf.xi, dy, true);
         const float s = 1.0f / dy.A[0];
@@ -935,7 +986,7 @@ __device__ __forceinline__ void efield_f32(const CellIn& c, const CellF& cf, con
         for (int i = 0; i < 3; i++)
             Ef[i] = (cf.etat * cf.Es[i] + ab * uf[i] + dy.A[2] * uxEs[i] + dy.A[3] * cf.B[i] + dy.A[5] * uxB[i]) * s;
         dE_dynamo<float>(dy.A, dy.Ad, Wf, uf, Ef, cf.Es, cf.B, dE);
-    } else if (c.emode == 1) {
+    } else if (emode == 1) {
         const float s = 1.0f / (Wf + cf.etat);
         const float A1 = cf.etat / (1.0f + cf.etat * Wf);
         const float Esu = cf.Es[0] * uf[0] + cf.Es[1] * uf[1] + cf.Es[2] * uf[2];
@@ -1023,7 +1074,7 @@ __device__ __forceinline__ bool newton_dir_f32(const CellIn& c, const CellF& cf,
     const float uu = uf[0] * uf[0] + uf[1] * uf[1] + uf[2] * uf[2];
     const float Wf = sqrtf(1.0f + uu), iWf = 1.0f / Wf;
     float Ef[3], dE[3][3];
-    efield_f32(c, cf, uf, Wf, iWf, Ef, dE);
+    efield_f32(c.emode, cf, uf, Wf, iWf, Ef, dE);
     // f scaled by 2^-k with 2^k <= M < 2^(k+1): the exponent field of M, read as an integer
     const int ek = (int)(mag_hi(e.M) >> 20);
     const bool scale = ek >= 1 && ek <= 2045;
@@ -1056,7 +1107,7 @@ __device__ __forceinline__ bool newton_step_f32(const CellIn& c, const CellF& cf
     const float uu = uf[0] * uf[0] + uf[1] * uf[1] + uf[2] * uf[2];
     const float Wf = sqrtf(1.0f + uu), iWf = 1.0f / Wf;
     float Ef[3], dE[3][3];
-    efield_f32(c, cf, uf, Wf, iWf, Ef, dE);
+    efield_f32(c.emode, cf, uf, Wf, iWf, Ef, dE);
     const float U = 0.5f * (Ef[0] * Ef[0] + Ef[1] * Ef[1] + Ef[2] * Ef[2] + cf.B[0] * cf.B[0] + cf.B[1] * cf.B[1] +
                             cf.B[2] * cf.B[2]);
     const float Sf[3] = {d2f_int(c.S[0]), d2f_int(c.S[1]), d2f_int(c.S[2])};
@@ -1115,76 +1166,139 @@ __device__ __forceinline__ dw dw_of(double x)
     return {h, (whi >> 31) ? -l : l};
 }
 
-__device__ __forceinline__ double dw_to_double(dw x) { return f2d_int(x.hi) + f2d_int(x.lo); }
-
-__device__ __forceinline__ dw dw_dot3(const dw* a, const dw* b)
+// a finite float widened on the integer pipe without f2d_int's infinities and NaN
+// (denormals and zero give zero)
+__device__ __forceinline__ double f2d_finite(float v)
 {
-    return dw_add(dw_add(dw_mul(a[0], b[0]), dw_mul(a[1], b[1])), dw_mul(a[2], b[2]));
+    const unsigned f = __float_as_uint(v);
+    const bool z = (f & 0x7f800000u) == 0u;
+    const unsigned hi = ((f & 0x7fffffffu) >> 3) + 0x38000000u;
+    return __hiloint2double((int)((f & 0x80000000u) | (z ? 0u : hi)), (int)(z ? 0u : f << 29));
 }
 
-// (a x b)_i = a_j b_k - a_k b_j
+// (an infinite or NaN hi keeps that; its lo is NaN or finite)
+__device__ __forceinline__ double dw_to_double(dw x) { return f2d_int(x.hi) + f2d_int(x.lo); }
+// the same of a finite value
+__device__ __forceinline__ double dw_finite(dw x) { return f2d_finite(x.hi) + f2d_finite(x.lo); }
+
+// the sums of products below gather the products' errors and renormalise once
+__device__ __forceinline__ dw dw_dot3(const dw* a, const dw* b)
+{
+    return dw_norm(dw_add_raw(dw_add_raw(dw_mul_raw(a[0], b[0]), dw_mul_raw(a[1], b[1])), dw_mul_raw(a[2], b[2])));
+}
+
+// (a x b)_i = a_j b_k - a_k b_j, not renormalised
+__device__ __forceinline__ dw dw_cross_raw(const dw* a, const dw* b, int i)
+{
+    const int j = (i + 1) % 3, k = (i + 2) % 3;
+    return dw_add_raw(dw_mul_raw(a[j], b[k]), dw_neg(dw_mul_raw(a[k], b[j])));
+}
+
+// (a x b)_i, renormalised
 __device__ __forceinline__ dw dw_cross(const dw* a, const dw* b, int i)
 {
     const int j = (i + 1) % 3, k = (i + 2) % 3;
     return dw_sub(dw_mul(a[j], b[k]), dw_mul(a[k], b[j]));
 }
 
+// the dot product with every term renormalised
+__device__ __forceinline__ dw dw_dot3_each(const dw* a, const dw* b)
+{
+    return dw_add(dw_add(dw_mul(a[0], b[0]), dw_mul(a[1], b[1])), dw_mul(a[2], b[2]));
+}
+
+// The per-cell constants of the solve as double-words, split from FP64 once per cell on
+// the integer pipe (a split takes 25 instructions and a residual uses 16 of them).
+struct CellDW {
+    dw D, S[3], B[3], Es[3], et;          // undensitised orthonormal components, eta_t
+    dw tD, B2h, Digh, etEs[3];            // tau + D, |B|^2 / 2, D / Gamma_hat, eta_t E*
+    dw igh;
+    int emode;                            // 0: E held fixed, 1: resistive
+};
+
+__device__ __forceinline__ CellDW cell_dw(const CellIn& c)
+{
+    CellDW d;
+    d.D = dw_of(c.D);
+    d.et = dw_of(c.etat);
+    d.igh = dw_of(c.igh);
+    d.emode = c.emode;
+    d.tD = dw_of(c.tD);
+    d.B2h = dw_of(c.B2h);
+    d.Digh = dw_of(c.Digh);
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        d.S[i] = dw_of(c.S[i]);
+        d.B[i] = dw_of(c.B[i]);
+        d.Es[i] = dw_of(c.Es[i]);
+        d.etEs[i] = dw_of(c.etEs[i]);
+    }
+    return d;
+}
+
 // The residual f = w_t u - S + E x B of evaluate() in double-word arithmetic, for the
-// resistive and E-fixed forms of E(u) (emode 1 and 0).  The per-cell constants are
-// split from their FP64 values on the integer pipe.  Outputs in binary32: f (each
+// resistive and E-fixed forms of E(u) (emode 1 and 0).  Outputs in binary32: f (each
 // accurate to ~1e-14 of the momentum scale), w_t, tau + D - U and the scale M.
 struct EvalDW {
     float f[3], wt, base, M;
 };
 
 // W, E(u) and w_t of the last double-word evaluation, kept when the residual there
-// accepts the root (double-word acceptance)
+// accepts the root (double-word acceptance), and its momentum scale
 struct DwRoot {
     dw W, wt, E[3];
+    float M;
 };
 
-template <bool KEEP = false>
-__device__ __forceinline__ void evaluate_dw(const CellIn& c, const dw* u, EvalDW& o, DwRoot* r = nullptr)
+// KEEP: the evaluation may accept the root (ACC), whose value it then carries: every term
+// is renormalised.  Without KEEP the FP64 residual decides, and sums of products gather
+// their errors and renormalise once (a quarter fewer instructions, the same accuracy).
+template <bool KEEP>
+__device__ __forceinline__ void evaluate_dw(const CellDW& c, const dw* u, EvalDW& o, DwRoot* r)
 {
-    dw S[3], B[3], E[3];
-#pragma unroll
-    for (int i = 0; i < 3; i++) {
-        S[i] = dw_of(c.S[i]);
-        B[i] = dw_of(c.B[i]);
-    }
-    const dw Wsq = dw_add_f(dw_add(dw_add(dw_sqr(u[0]), dw_sqr(u[1])), dw_sqr(u[2])), 1.0f);
+    dw E[3];
+    const dw Wsq = KEEP ? dw_add_f(dw_add(dw_add(dw_sqr(u[0]), dw_sqr(u[1])), dw_sqr(u[2])), 1.0f)
+                        : dw_add_f(dw_dot3(u, u), 1.0f);
     const dw W = dw_sqrt(Wsq);
     if (c.emode == 1) {
         // A_0 E = eta_t E* + A_1 (E*.u) u - u x B, A_0 = W + eta_t, A_1 = eta_t/(1 + eta_t W)
-        const dw et = dw_of(c.etat);
-        dw Es[3];
-#pragma unroll
-        for (int i = 0; i < 3; i++) Es[i] = dw_of(c.Es[i]);
-        const dw iWe = dw_rcp(dw_add(W, et));
-        const dw A1 = dw_mul(et, dw_rcp(dw_add_f(dw_mul(et, W), 1.0f)));
-        const dw ae = dw_mul(A1, dw_dot3(Es, u));
+        const dw iWe = dw_rcp(dw_add(W, c.et));
+        const dw A1 = dw_mul(c.et, dw_rcp(dw_add_f(dw_mul(c.et, W), 1.0f)));
+        const dw ae = dw_mul(A1, KEEP ? dw_dot3_each(c.Es, u) : dw_dot3(c.Es, u));
 #pragma unroll
         for (int i = 0; i < 3; i++)
-            E[i] = dw_mul(dw_sub(dw_add(dw_of(c.etEs[i]), dw_mul(ae, u[i])), dw_cross(u, B, i)), iWe);
+            E[i] = dw_mul(KEEP ? dw_sub(dw_add(c.etEs[i], dw_mul(ae, u[i])), dw_cross(u, c.B, i))
+                               : dw_norm(dw_add_raw(dw_add_raw(c.etEs[i], dw_mul_raw(ae, u[i])),
+                                                    dw_neg(dw_cross_raw(u, c.B, i)))), iWe);
     } else {
 #pragma unroll
-        for (int i = 0; i < 3; i++) E[i] = dw_of(c.Es[i]);
+        for (int i = 0; i < 3; i++) E[i] = c.Es[i];
     }
     // U = |E|^2/2 + |B|^2/2;  w_t = (W (tau + D - U) - D/Gamma_hat) / (W^2 - 1/Gamma_hat)
-    const dw U = dw_add(dw_scale(dw_dot3(E, E), 0.5f), dw_of(c.B2h));
-    const dw base = dw_sub(dw_of(c.tD), U);
-    const dw wt = dw_mul(dw_sub(dw_mul(W, base), dw_of(c.Digh)), dw_rcp(dw_sub(Wsq, dw_of(c.igh))));
+    const dw U = dw_add(dw_scale(KEEP ? dw_dot3_each(E, E) : dw_dot3(E, E), 0.5f), c.B2h);
+    const dw base = dw_sub(c.tD, U);
+    const dw wt = dw_mul(KEEP ? dw_sub(dw_mul(W, base), c.Digh)
+                              : dw_norm(dw_add_raw(dw_mul_raw(W, base), dw_neg(c.Digh))), dw_rcp(dw_sub(Wsq, c.igh)));
     float M = 0.0f;
 #pragma unroll
     for (int i = 0; i < 3; i++) {
-        const dw x = dw_cross(E, B, i);
-        const dw w = dw_mul(wt, u[i]);
-        o.f[i] = dw_add(dw_sub(w, S[i]), x).hi;
-        M = fmaxf(M, fmaxf(fabsf(S[i].hi), fmaxf(fabsf(x.hi), fabsf(w.hi))));
+        dw x, w;
+        if (KEEP) {
+            x = dw_cross(E, c.B, i);
+            w = dw_mul(wt, u[i]);
+            o.f[i] = dw_add(dw_sub(w, c.S[i]), x).hi;
+        } else {
+            x = dw_cross_raw(E, c.B, i);
+            w = dw_mul_raw(wt, u[i]);
+            const dw s = dw_add_raw(dw_add_raw(w, dw_neg(c.S[i])), x);
+            o.f[i] = __fadd_rn(s.hi, s.lo);
+        }
+        M = fmaxf(M, fmaxf(fabsf(c.S[i].hi), fmaxf(fabsf(x.hi), fabsf(w.hi))));
     }
     o.wt = wt.hi;
     o.base = base.hi;
     o.M = M;
+    r->M = M;
     if (KEEP) {
         r->W = W;
         r->wt = wt;
@@ -1193,78 +1307,152 @@ __device__ __forceinline__ void evaluate_dw(const CellIn& c, const dw* u, EvalDW
     }
 }
 
-// Newton corrections from the double-word residual with the FP32 Jacobian (the
-// direction of newton_dir_f32, here at the double-word velocity), at most `nit`
-// evaluations.  It stops once |f| <= tol M / 4 in double-word arithmetic, or after a
-// step |dx|^2 <= tol max(|u|^2, 1) / 100: the FP32 Jacobian contracts the error by
-// ~1e-6 per step and the quadratic term is ~|dx|^2, so the residual after such a step
-// is already below the tolerance and the FP64 residual can accept it directly.  Steps
-// are taken only when finite and within the step bound; u (FP64) receives the result
-// only if it is finite.
+// 1/x by the hardware's approximate reciprocal (2^-23; only the FP32 Newton direction
+// takes it, whose other roundings are as large)
+__device__ __forceinline__ float rcp_approx(float x) { return __fdividef(1.0f, x); }
+
+// K = -(J / w_t)^{-1} / w_t in FP32 at the velocity uf (so that dx = K f): E(u) and
+// dE_i/du_j as efield_f32, J as solve_f32; base = tau + D - U.  False when singular.
+__device__ __forceinline__ bool newton_inverse_f32(const CellDW& c, const float* uf, float wt, float base, float* K)
+{
+    const float uu = uf[0] * uf[0] + uf[1] * uf[1] + uf[2] * uf[2];
+    const float iWf = rsqrtf(1.0f + uu), Wf = (1.0f + uu) * iWf;
+    const float B[3] = {c.B[0].hi, c.B[1].hi, c.B[2].hi};
+    const float scf = rcp_approx(wt);
+    const float basef = base * scf;
+    const float idenf = rcp_approx(uu + 1.0f - c.igh.hi);
+    float J[3][3];
+    if (c.emode == 1) {
+        const float Es[3] = {c.Es[0].hi, c.Es[1].hi, c.Es[2].hi}, et = c.et.hi;
+        const float s = rcp_approx(Wf + et);
+        const float A1 = et * rcp_approx(1.0f + et * Wf);
+        const float Esu = Es[0] * uf[0] + Es[1] * uf[1] + Es[2] * uf[2];
+        const float ae = A1 * Esu;
+        const float Ef[3] = {(et * Es[0] + ae * uf[0] - (uf[1] * B[2] - uf[2] * B[1])) * s,
+                             (et * Es[1] + ae * uf[1] - (uf[2] * B[0] - uf[0] * B[2])) * s,
+                             (et * Es[2] + ae * uf[2] - (uf[0] * B[1] - uf[1] * B[0])) * s};
+        const float a2 = A1 * ae * iWf;
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const float ui = uf[j] * iWf;
+            float dE[3];
+#pragma unroll
+            for (int i = 0; i < 3; i++)
+                dE[i] = -Ef[i] * ui + uf[i] * (A1 * Es[j] - a2 * uf[j]) + (i == j ? ae : 0.0f);
+            const int j1 = (j + 1) % 3, j2 = (j + 2) % 3;
+            dE[j1] += B[j2];   // -(e_j x B)
+            dE[j2] -= B[j1];
+#pragma unroll
+            for (int i = 0; i < 3; i++) dE[i] *= s;
+            const float dU = Ef[0] * dE[0] + Ef[1] * dE[1] + Ef[2] * dE[2];
+            const float dw_ = (basef * ui - Wf * dU * scf - 2.0f * uf[j]) * idenf;
+            J[0][j] = uf[0] * dw_ + (dE[1] * B[2] - dE[2] * B[1]) * scf;
+            J[1][j] = uf[1] * dw_ + (dE[2] * B[0] - dE[0] * B[2]) * scf;
+            J[2][j] = uf[2] * dw_ + (dE[0] * B[1] - dE[1] * B[0]) * scf;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const float dw_ = (basef * uf[j] * iWf - 2.0f * uf[j]) * idenf;
+#pragma unroll
+            for (int i = 0; i < 3; i++) J[i][j] = uf[i] * dw_;
+        }
+    }
+    J[0][0] += 1.0f; J[1][1] += 1.0f; J[2][2] += 1.0f;
+    const float c00 = J[1][1] * J[2][2] - J[1][2] * J[2][1];
+    const float c01 = J[1][2] * J[2][0] - J[1][0] * J[2][2];
+    const float c02 = J[1][0] * J[2][1] - J[1][1] * J[2][0];
+    const float det = J[0][0] * c00 + J[0][1] * c01 + J[0][2] * c02;
+    if (!(fabsf(det) > 1e-30f)) return false;
+    const float id = -scf * rcp_approx(det);
+    K[0] = c00 * id;
+    K[1] = (J[0][2] * J[2][1] - J[0][1] * J[2][2]) * id;
+    K[2] = (J[0][1] * J[1][2] - J[0][2] * J[1][1]) * id;
+    K[3] = c01 * id;
+    K[4] = (J[0][0] * J[2][2] - J[0][2] * J[2][0]) * id;
+    K[5] = (J[0][2] * J[1][0] - J[0][0] * J[1][2]) * id;
+    K[6] = c02 * id;
+    K[7] = (J[0][1] * J[2][0] - J[0][0] * J[2][1]) * id;
+    K[8] = (J[0][0] * J[1][1] - J[0][1] * J[1][0]) * id;
+    return true;
+}
+
+// Newton corrections of the double-word velocity u from the double-word residual with
+// the FP32 Jacobian, at most `nit` evaluations.  Without ACC it stops with the step from a
+// residual |f| <= tol M / 4 in double-word arithmetic (at the start itself: without a
+// step), or after a step |dx|^2 <= 1e-5 tol max(|u|^2, 1): the FP32 Jacobian contracts the
+// error by ~1e-6 per step and the quadratic term is ~|dx|^2, so such a step (1e-9 at the
+// default tolerance) leaves ~1e-15 and the FP64 residual can accept it directly.  (Ending
+// at 3e-8 left up to 2e-14 in a cold first step; a start from the extrapolated history
+// takes as many evaluations either way.)  After a step |dx| <= 1e-5 max(|u|, 1) the next
+// one reuses the inverse Jacobian: it has changed by that much, and the next step is that
+// much smaller again.  Steps are taken only when finite and within the step bound.
 //
 // ACC (double-word acceptance, for tolerances of 1e-11 and above): the double-word
 // residual itself accepts the root.  It is accurate to ~1e-14 of the momentum scale,
 // a few hundred times below tol M / 4 there, so |f| <= tol M / 4 in double-word
 // arithmetic bounds the exact residual by the tolerance.  The small-step exit is then
-// skipped (the next evaluation decides), and on acceptance u, W, 1/W, w_t and E(u)
-// are written to e from the double-word values; the return value says whether that
-// happened (else the FP64 residual decides, as without ACC).
+// skipped (the next evaluation decides), and on acceptance r holds W, w_t and E(u) there;
+// the return value says whether that happened (else the FP64 residual decides, as without
+// ACC).
 constexpr int kDwEvals = 4;   // most double-word residual evaluations per solve
 constexpr unsigned kHi1e10 = 0x4202A05Fu;   // high word of 1e10 (the bound on W)
 
 template <bool ACC>
-__device__ __forceinline__ bool newton_refine_dw(const CellIn& c, const CellF& cf, double* u, float tol, int nit,
-                                                 Eval* e)
+__device__ __forceinline__ bool newton_refine_dw(const CellDW& c, dw* u, float tol, int nit, DwRoot* r)
 {
-    dw ud[3];
-#pragma unroll
-    for (int i = 0; i < 3; i++) ud[i] = dw_of(u[i]);
-    bool moved = false;
+    float K[9];
+    bool reuse = false;
+#pragma unroll 1
     for (int k = 0; k < nit; k++) {
         EvalDW ed;
-        DwRoot rt;
-        evaluate_dw<ACC>(c, ud, ed, &rt);
-        if (!(ed.M > 0.0f) || !(ed.M < 1e30f) || !(ed.wt > 0.0f)) break;
+        evaluate_dw<ACC>(c, u, ed, r);
+        if (!(ed.M > 0.0f) || !(ed.M < 1e30f) || !(ed.wt > 0.0f)) return false;
         const float fm = fmaxf(fabsf(ed.f[0]), fmaxf(fabsf(ed.f[1]), fabsf(ed.f[2])));
-        if (fm <= 0.25f * tol * ed.M) {   // also false for NaN
-            if (ACC && rt.W.hi < 1e10f) {
-                const dw iW = dw_rcp(rt.W);
+        const bool small = fm <= 0.25f * tol * ed.M;   // (false for NaN)
+        if (small && (ACC || k == 0)) return ACC && r->W.hi < 1e10f;
+        const float uf[3] = {u[0].hi, u[1].hi, u[2].hi};
+        float dx[3];
+        if (ACC) {
+            // (the direction is formed anew each time and with full FP32 divisions: the
+            // accepted root carries its rounding, to tol / 4)
+            const float uq = uf[0] * uf[0] + uf[1] * uf[1] + uf[2] * uf[2];
+            const float Wf = sqrtf(1.0f + uq), iWf = 1.0f / Wf;
+            CellF cf;
 #pragma unroll
-                for (int i = 0; i < 3; i++) {
-                    u[i] = dw_to_double(ud[i]);
-                    e->E[i] = dw_to_double(rt.E[i]);
-                }
-                e->W = dw_to_double(rt.W);
-                e->iW = dw_to_double(iW);
-                e->wt = dw_to_double(rt.wt);
-                return true;
+            for (int i = 0; i < 3; i++) {
+                cf.Es[i] = c.Es[i].hi;
+                cf.B[i] = c.B[i].hi;
             }
-            break;
-        }
-        const float uf[3] = {ud[0].hi, ud[1].hi, ud[2].hi};
-        const float uu = uf[0] * uf[0] + uf[1] * uf[1] + uf[2] * uf[2];
-        const float Wf = sqrtf(1.0f + uu), iWf = 1.0f / Wf;
-        float Ef[3], dE[3][3];
-        efield_f32(c, cf, uf, Wf, iWf, Ef, dE);
-        const float iM = 1.0f / ed.M;
-        const float fs[3] = {ed.f[0] * iM, ed.f[1] * iM, ed.f[2] * iM};
-        float y[3];
-        if (!solve_f32(cf, uf, Wf, iWf, uu, Ef, dE, ed.wt, ed.base, fs, y)) break;
-        const float dx[3] = {y[0] * ed.M, y[1] * ed.M, y[2] * ed.M};
-        const float nx2 = dx[0] * dx[0] + dx[1] * dx[1] + dx[2] * dx[2];
-        if (!(nx2 <= 1e4f * fmaxf(1.0f, uu))) break;   // also rejects NaN
+            cf.etat = c.et.hi;
+            cf.xi = 0.0f;
+            cf.igh = c.igh.hi;
+            float Ef[3], dE[3][3];
+            if (c.emode == 1) efield_f32(1, cf, uf, Wf, iWf, Ef, dE);
+            else efield_f32(0, cf, uf, Wf, iWf, Ef, dE);
+            const float iM = 1.0f / ed.M;
+            const float fs[3] = {ed.f[0] * iM, ed.f[1] * iM, ed.f[2] * iM};
+            float y[3];
+            if (!solve_f32(cf, uf, Wf, iWf, uq, Ef, dE, ed.wt, ed.base, fs, y)) return false;
 #pragma unroll
-        for (int i = 0; i < 3; i++) ud[i] = dw_add_f(ud[i], dx[i]);
-        moved = true;
-        if (!ACC && nx2 <= 0.01f * tol * fmaxf(1.0f, uu)) break;
-    }
-    if (moved) {
-        const double v[3] = {dw_to_double(ud[0]), dw_to_double(ud[1]), dw_to_double(ud[2])};
-        if (finite_int(v[0]) && finite_int(v[1]) && finite_int(v[2])) {
-            u[0] = v[0];
-            u[1] = v[1];
-            u[2] = v[2];
+            for (int i = 0; i < 3; i++) dx[i] = y[i] * ed.M;
+        } else {
+            // (a last step from a residual below the tolerance costs little with the inverse at
+            // hand, and leaves the double-words' own error)
+            if (!reuse && !small && !newton_inverse_f32(c, uf, ed.wt, ed.base, K)) return false;
+            // scaled to the momentum scale, so that no product of small numbers underflows
+            const float iM = rcp_approx(ed.M);
+            const float fs[3] = {ed.f[0] * iM, ed.f[1] * iM, ed.f[2] * iM};
+#pragma unroll
+            for (int i = 0; i < 3; i++) dx[i] = (K[3 * i] * fs[0] + K[3 * i + 1] * fs[1] + K[3 * i + 2] * fs[2]) * ed.M;
         }
+        const float uu = fmaxf(1.0f, uf[0] * uf[0] + uf[1] * uf[1] + uf[2] * uf[2]);
+        const float nx2 = dx[0] * dx[0] + dx[1] * dx[1] + dx[2] * dx[2];
+        if (!(nx2 <= 1e4f * uu)) return false;   // also rejects NaN
+#pragma unroll
+        for (int i = 0; i < 3; i++) u[i] = dw_add_f(u[i], dx[i]);
+        if (!ACC && (small || nx2 <= 1e-5f * tol * uu)) return false;
+        reuse = nx2 <= 1e-10f * uu;
     }
     return false;
 }
@@ -1289,7 +1477,25 @@ __device__ __forceinline__ int newton_solve(const CellIn& c, double* u, Eval& e,
         // Newton corrections from the double-word residual; the FP64 residual below
         // then accepts the root (or, with ACC, the double-word one already did), or the
         // FP64 iteration continues from there
-        if (newton_refine_dw<ACC>(c, cf, u, tolf, kDwEvals, &e)) return 0;
+        dw ud[3];
+#pragma unroll
+        for (int i = 0; i < 3; i++) ud[i] = dw_of(u[i]);
+        DwRoot rt;
+        const bool acc = newton_refine_dw<ACC>(cell_dw(c), ud, tolf, kDwEvals, &rt);
+        const double v[3] = {dw_to_double(ud[0]), dw_to_double(ud[1]), dw_to_double(ud[2])};
+        if (finite_int(v[0]) && finite_int(v[1]) && finite_int(v[2])) {
+            u[0] = v[0];
+            u[1] = v[1];
+            u[2] = v[2];
+        }
+        if (acc) {
+#pragma unroll
+            for (int i = 0; i < 3; i++) e.E[i] = dw_to_double(rt.E[i]);
+            e.W = dw_to_double(rt.W);
+            e.iW = dw_to_double(dw_rcp(rt.W));
+            e.wt = dw_to_double(rt.wt);
+            return 0;
+        }
         has1 = false;
     } else if (tol < 1e-11) {
         F3 un;

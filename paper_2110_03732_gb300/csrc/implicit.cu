@@ -7,12 +7,15 @@
 
 namespace grmhd {
 
-// Five blocks per SM (96 registers, about 1 KB of spills): against four (128 registers)
-// the mixed-precision and metric instances ran 1.5-4 % faster (512^2 vortex mixed 58.1 ->
-// 57.3 us, 128^3 star mixed 398 -> 381 us, FP64 455 -> 442 us per launch); the flat FP64
-// instance is unchanged (79.3 us).
+// Seven blocks per SM (72 registers, 130-200 B of spills): the solve waits on its loads and
+// on dependent arithmetic, so more warps pay until the spills do not.  us per launch at
+// five / six / seven / eight blocks: 512^2 vortex FP64 65.7 / 61.7 / 60.3 / 61.2, mixed 44.6 /
+// 44.3 / 42.4 / 43.4; 96^3 star mixed 147 / 144 / 148 / 149.  (With the FP64 iteration inlined
+// in the kernel and the constants split at every residual it took 79.6 and 57.3 us at five
+// blocks, and 168 us; 128^3 star FP64 398 us, 277 now.)  The arguments are grid constants because implicit_general takes
+// them by reference: as plain parameters every thread copied them to its stack.
 template <bool M, bool ACC>
-__global__ void __launch_bounds__(128, 5) k_implicit(Dims g, ImpArgs a)
+__global__ void __launch_bounds__(128, 7) k_implicit(const __grid_constant__ Dims g, const __grid_constant__ ImpArgs a)
 {
     grid_dep_sync();
     const long long tot = (long long)g.n[0] * g.n[1] * g.n[2];
@@ -21,9 +24,10 @@ __global__ void __launch_bounds__(128, 5) k_implicit(Dims g, ImpArgs a)
         implicit_item<M, false, ACC>(g, a, t);
 }
 
-// the same solve with cell-centred q_B (GLM variant, Sec. 3.1)
+// the same solve with cell-centred q_B (GLM variant, Sec. 3.1); eight blocks: 384^2 vortex
+// 40.8 / 39.8 / 39.1 / 37.1 us at five to eight
 template <bool M>
-__global__ void __launch_bounds__(128, 4) k_implicit_cc(Dims g, ImpArgs a)
+__global__ void __launch_bounds__(128, 8) k_implicit_cc(const __grid_constant__ Dims g, const __grid_constant__ ImpArgs a)
 {
     grid_dep_sync();
     const long long tot = (long long)g.n[0] * g.n[1] * g.n[2];

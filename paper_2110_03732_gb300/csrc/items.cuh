@@ -13,11 +13,58 @@ namespace grmhd {
 // implicit step (Sec. 2.4): item t = interior cell t (x fastest)
 // ---------------------------------------------------------------------------
 
+// The outputs of a solved cell: primitives (FP64, and on the mixed path their FP32 copy
+// from the caller's f32 = rho, u^1..3, p, E^1..3, q_B^1..3), the stiff rate R, the solved
+// q_E and the history (uh: the FP32 orthonormal velocity, or NULL).  u and E orthonormal;
+// qEs the stage base's q_E.
+template <bool M>
+__device__ __forceinline__ void implicit_store(const ImpArgs& a, long long id, double rho, double pres,
+                                               const double* u, const double* E, double ip2, double p4,
+                                               const double* qEs, const float* f32, const float* uh)
+{
+    a.prim.p[0][id] = rho;
+    a.prim.p[4][id] = pres;
+    if (a.p32.p[0]) {
+#pragma unroll
+        for (int v = 0; v < 11; v++) a.p32.p[v][id] = f32[v];
+    }
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        a.prim.p[1 + i][id] = M ? u[i] * ip2 : u[i];
+        a.prim.p[5 + i][id] = M ? E[i] * ip2 : E[i];
+        const double qEn = M ? p4 * E[i] : E[i];
+        if (a.R.p[0]) a.R.p[i][id] = a.stiff ? (qEn - qEs[i]) * a.ia_dt : 0.0;
+        if (a.qE_out.p[0]) a.qE_out.p[i][id] = qEn;
+        if (a.hs[0] && uh) {
+            a.hd[i][id] = uh[i] - a.hs[i][id];
+            a.hs[i][id] = uh[i];
+        }
+    }
+}
+
+// the FP32 copies of a cell's primitives, converted on the integer pipe (a hardware
+// conversion issues on the FP64 pipe)
+template <bool M>
+__device__ __forceinline__ void implicit_f32(double rho, double pres, const double* u, const double* E, double ip2,
+                                             float* f32)
+{
+    f32[0] = d2f_int(rho);
+    f32[4] = d2f_int(pres);
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        f32[1 + i] = d2f_int(M ? u[i] * ip2 : u[i]);
+        f32[5 + i] = d2f_int(M ? E[i] * ip2 : E[i]);
+    }
+}
+
+// The general solve of one cell (cells that implicit_item's direct path does not accept,
+// and the dynamo form): a call, so that its FP64 iteration takes neither registers nor
+// instruction-cache room from the direct path.
 // CC: the magnetic field is cell-centred (a.bf holds cell q_B, GLM variant) instead of
 // staggered on faces.  ACC: the mixed-precision path, whose double-word residual
 // accepts the root (newton_refine_dw)
-template <bool M, bool CC = false, bool ACC = false>
-__device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, long long t)
+template <bool M, bool CC, bool ACC>
+__device__ __noinline__ void implicit_general(const Dims& g, const ImpArgs& a, long long t)
 {
     // flat metric: alpha = psi = 1 known at compile time
     const double* __restrict__ psi = M ? a.psi : nullptr;
@@ -29,8 +76,6 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
     const int kmax = a.kmax;
     const P8& prim = a.prim;
     const P3& R = a.R;
-    const P3& qE_out = a.qE_out;
-    const F11& p32 = a.p32;
     unsigned long long* nfail = a.nfail;
     int c[3];
     interior_coords(g, t, c);
@@ -67,7 +112,6 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
     // over steps, kept in FP32: it is only a start) when the history is kept, else the
     // latest primitives
     const bool hist = a.hs[0] != nullptr;
-    float hsv[3] = {0.0f, 0.0f, 0.0f};
     F3 ust = {{0.0f, 0.0f, 0.0f}};
     if (a.atm && ci.D < a.d_atm) {
         atmo = true;   // (its history is left as it is)
@@ -76,8 +120,7 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
 #pragma unroll
         for (int i = 0; i < 3; i++) {
             if (hist) {
-                hsv[i] = a.hs[i][id];
-                ust.x[i] = hsv[i] + a.hd[i][id];
+                ust.x[i] = a.hs[i][id] + a.hd[i][id];
                 u[i] = f2d_int(ust.x[i]);
             } else {
                 u[i] = p2 * prim.p[1 + i][id];
@@ -116,33 +159,147 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
         rho = ci.D * iW;
         pres = (e.wt * iW - rho) * g.igh;
     }
-    prim.p[0][id] = rho;
-    prim.p[4][id] = pres;
-    if (p32.p[0]) {
-        // FP32 copy for the mixed-precision explicit kernels, with the densitised
-        // cell-centred q_B of the stage
-        // (converted on the integer pipe: a hardware conversion issues on the FP64 pipe)
-        p32.p[0][id] = d2f_int(rho);
-        p32.p[4][id] = d2f_int(pres);
-#pragma unroll
-        for (int i = 0; i < 3; i++) {
-            p32.p[1 + i][id] = d2f_int(u[i] * ip2);
-            p32.p[5 + i][id] = d2f_int(e.E[i] * ip2);
-            p32.p[8 + i][id] = d2f_int(ci.B[i] * p4);
-        }
-    }
+    float f32[11], uh[3];
+    implicit_f32<M>(rho, pres, u, e.E, ip2, f32);
 #pragma unroll
     for (int i = 0; i < 3; i++) {
-        prim.p[1 + i][id] = u[i] * ip2;
-        prim.p[5 + i][id] = e.E[i] * ip2;
-        const double qEn = p4 * e.E[i];
-        if (R.p[0]) R.p[i][id] = a.stiff ? (qEn - qEs[i]) * a.ia_dt : 0.0;
-        if (qE_out.p[0]) qE_out.p[i][id] = qEn;
-        if (hist && !atmo) {
-            const float un = d2f_int(u[i]);
-            a.hd[i][id] = un - hsv[i];
-            a.hs[i][id] = un;
+        f32[8 + i] = d2f_int(ci.B[i] * p4);
+        uh[i] = d2f_int(u[i]);
+    }
+    implicit_store<M>(a, id, rho, pres, u, e.E, ip2, p4, qEs, f32, atmo ? nullptr : uh);
+}
+
+// One cell: the direct path takes the double-word Newton corrections from the kept start
+// and accepts their root by the FP64 residual (ACC: the double-word one); atmosphere cells
+// are written at once; everything else is implicit_general's.  The FP64 inputs are split
+// into double-words as they are loaded and loaded again for the FP64 residual (L1 holds
+// them), so that only one form is live during the corrections.
+template <bool M, bool CC = false, bool ACC = false>
+__device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, long long t)
+{
+    int c[3];
+    interior_coords(g, t, c);
+    const long long id = lin(g, c[0], c[1], c[2]);
+    if ((__double_as_longlong(a.xi) << 1) != 0) {   // the dynamo form (xi != 0)
+        implicit_general<M, CC, ACC>(g, a, t);
+        return;
+    }
+    const double* __restrict__ psi = M ? a.psi : nullptr;
+    const double* __restrict__ alp = M ? a.alp : nullptr;
+    const double ps = psi ? psi[id] : 1.0;
+    const double p2 = ps * ps, p4 = p2 * p2, ip2 = M ? rcp_pos(p2) : 1.0, ip4 = ip2 * ip2, ip6 = ip4 * ip2;
+    auto qE = [&](int i) { return a.qb.p[5 + i][id]; };
+    auto qB = [&](int i) { return CC ? a.bf.p[i][id] : cell_qB_in(g, a.bf.p[i], i, c, id); };
+    auto mul = [](double x, double f) { return M ? x * f : x; };
+    const double D = mul(a.qb.p[0][id], ip6);
+    if (a.atm && D < a.d_atm) {
+        // atmosphere: rest state at the floor density and pressure, E kept; its history is
+        // left as it is
+        const double z[3] = {0.0, 0.0, 0.0};
+        double q[3], Es[3];
+        float f32[11];
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            q[i] = qE(i);
+            Es[i] = mul(q[i], ip4);
         }
+        if (a.p32.p[0]) {
+            implicit_f32<M>(a.rho_atm, a.p_atm, z, Es, ip2, f32);
+#pragma unroll
+            for (int i = 0; i < 3; i++) f32[8 + i] = d2f_int(mul(mul(qB(i), ip4), p4));
+        }
+        implicit_store<M>(a, id, a.rho_atm, a.p_atm, z, Es, ip2, p4, q, f32, nullptr);
+        return;
+    }
+    // the start: this stage's last root plus its last change, or the latest velocity
+    const bool hist = a.hs[0] != nullptr;
+    dw ud[3];
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        if (hist) {
+            ud[i] = dw_make(a.hs[i][id] + a.hd[i][id]);
+        } else {
+            ud[i] = dw_of(mul(a.prim.p[1 + i][id], p2));
+        }
+        if (!(fabsf(ud[i].hi) < 1e30f)) ok = false;   // also NaN
+    }
+    const double et = a.eta ? a.eta[id] : a.eta_u;
+    // flat: eta / (a_ii dt) with the host's reciprocal, no division
+    const double etat = a.stiff ? (M ? et * rcp_pos(alp ? alp[id] : 1.0) * a.ia_dt : et * a.ia_dt) : -1.0;
+    const long long eb = __double_as_longlong(etat);
+    const int emode = (eb >= 0 && eb <= 0x7ff0000000000000ll) || eb == (long long)0x8000000000000000ull ? 1 : 0;
+    DwRoot rt;
+    rt.M = 0.0f;
+    bool acc;
+    float B32[3];
+    {
+        // the derived constants in FP64 (formed in double-word arithmetic they would add to
+        // the residual's error)
+        CellIn ci;
+        ci.D = D;
+        ci.tau = mul(a.qb.p[4][id], ip6);
+        ci.igh = g.igh;
+        ci.etat = etat;
+        ci.xi = 0.0;
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            ci.S[i] = mul(mul(a.qb.p[1 + i][id], ip6), ip2);
+            ci.Es[i] = mul(qE(i), ip4);
+            ci.B[i] = mul(qB(i), ip4);
+        }
+        cell_derive(ci);
+        CellDW cd = cell_dw(ci);
+        cd.igh = {a.ighf, a.ighl};
+#pragma unroll
+        for (int i = 0; i < 3; i++) B32[i] = cd.B[i].hi;
+        acc = ok && newton_refine_dw<ACC>(cd, ud, a.tolf, kDwEvals, &rt);
+    }
+    asm volatile("" ::: "memory");   // what follows loads its inputs anew
+    double u[3], q[3];
+    float f32[11], uh[3];
+    if (ACC) {
+        if (!acc) {
+            implicit_general<M, CC, ACC>(g, a, t);
+            return;
+        }
+        const double iW = dw_finite(dw_rcp(rt.W));
+        const double rho = mul(a.qb.p[0][id], ip6) * iW, pres = (dw_finite(rt.wt) * iW - rho) * g.igh;
+        double E[3];
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            u[i] = dw_finite(ud[i]);
+            uh[i] = d2f_int(u[i]);
+            E[i] = dw_finite(rt.E[i]);
+            q[i] = qE(i);
+        }
+        implicit_f32<M>(rho, pres, u, E, ip2, f32);
+#pragma unroll
+        for (int i = 0; i < 3; i++) f32[8 + i] = M ? d2f_int(mul(mul(qB(i), ip4), p4)) : B32[i];
+        implicit_store<M>(a, id, rho, pres, u, E, ip2, p4, q, f32, uh);
+    } else {
+        double S[3], Es[3], B[3];
+        const double Dn = mul(a.qb.p[0][id], ip6);
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            u[i] = dw_to_double(ud[i]);
+            S[i] = mul(mul(a.qb.p[1 + i][id], ip6), ip2);
+            q[i] = qE(i);
+            Es[i] = mul(q[i], ip4);
+            B[i] = mul(qB(i), ip4);
+        }
+        Accept e;
+        evaluate_accept(Dn, mul(a.qb.p[4][id], ip6), S, Es, B, etat, g.igh, emode, u, e);
+        const double fm = from_hi(max(mag_hi(e.f[0]), max(mag_hi(e.f[1]), mag_hi(e.f[2]))));
+        // (every comparison is false for a NaN)
+        if (!ok || !(rt.M > 0.0f) || !(fm <= a.tol * f2d_int(rt.M)) || !pos_int(e.wt) || !mag_below_int(e.W, kHi1e10)) {
+            implicit_general<M, CC, ACC>(g, a, t);
+            return;
+        }
+        const double rho = Dn * e.iW, pres = fma(e.wt, e.iW, -rho) * g.igh;
+#pragma unroll
+        for (int i = 0; i < 3; i++) uh[i] = d2f_int(u[i]);
+        implicit_store<M>(a, id, rho, pres, u, e.E, ip2, p4, q, f32, uh);
     }
 }
 

@@ -29,7 +29,7 @@ struct ImpArgs {
     double eta_u;
     double a_dt;            // a_ii dt (<= 0: E held fixed)
     double ia_dt;           // 1 / (a_ii dt) (0 when a_dt <= 0)
-    float ighf, xif;        // FP32 1/Gamma_hat and xi
+    float ighf, ighl, xif;  // 1/Gamma_hat as a double-word ighf + ighl, and FP32 xi
     P8 prim;                // in: Newton start; out: stage primitives
     P3 R;                   // stiff rates (or NULL)
     P3 qE_out;              // solved q_E (or NULL)
