@@ -62,7 +62,13 @@ enum { WL_IMP = 0, WL_FLUX = 1, WL_EMF = 4, WL_UPD = 7, WL_KINDS = 8 };
 constexpr int kAlign = 256;
 size_t rup(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
-// autotuner candidates: threads per block, items per chunk
+// autotuner candidates: threads per block, items per chunk.  The first is the default: one
+// chunk per block and small chunks, which the hardware spreads evenly (24 mixed-precision
+// boxes of 64 to 400 cells a side: 512-item chunks walked by at most 2048 threads per SM left
+// a nearly empty second round, 1.69 ms per step against 1.55).  Register bounds of the
+// mixed-precision kernels on that batch, us per launch: flux two blocks of 256 threads (128
+// registers) 68 + 73, three 91 + 86; EMF four 68, three 81, two 90; update eight 200, six
+// 217, five 228; 1.39 ms per step together.
 struct Cfg {
     int threads, items;
 };
@@ -110,7 +116,7 @@ __device__ __forceinline__ void flux_any_item(const ProbStage& ps, double* sm, l
 }
 
 template <int D, bool M, typename T>
-__global__ void __launch_bounds__(sizeof(T) == 8 ? Flux64<false, false>::NT : 256) kb_flux(const ProbStage* __restrict__ P, int s, int stage,
+__global__ void __launch_bounds__(sizeof(T) == 8 ? Flux64<false, false>::NT : 256, sizeof(T) == 8 ? 4 : 2) kb_flux(const ProbStage* __restrict__ P, int s, int stage,
                                               const Chunk* __restrict__ ch, int nch)
 {
     __shared__ double sm[sizeof(T) == 8 ? Flux64<false, false>::SM : 1];
@@ -135,7 +141,7 @@ __device__ __forceinline__ void emf_any_item(const ProbStage& ps, long long t)
 }
 
 template <int C, bool M, typename T>
-__global__ void __launch_bounds__(256) kb_emf(const ProbStage* __restrict__ P, int s, int stage,
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 4) kb_emf(const ProbStage* __restrict__ P, int s, int stage,
                                              const Chunk* __restrict__ ch, int nch)
 {
     for (int i = blockIdx.x; i < nch; i += gridDim.x) {
@@ -146,7 +152,7 @@ __global__ void __launch_bounds__(256) kb_emf(const ProbStage* __restrict__ P, i
 }
 
 template <bool M, bool F32>
-__global__ void __launch_bounds__(256) kb_update(const ProbStage* __restrict__ P, int s, int stage,
+__global__ void __launch_bounds__(256, F32 ? 8 : 4) kb_update(const ProbStage* __restrict__ P, int s, int stage,
                                                 const Chunk* __restrict__ ch, int nch)
 {
     for (int i = blockIdx.x; i < nch; i += gridDim.x) {
@@ -408,9 +414,7 @@ void fill_desc(grmhd_batch* b, int p, double dt)
 
 int grid_of(const grmhd_batch* b, int kind, int m)
 {
-    const int nch = b->cnt[kind][m];
-    const int cap = b->nsm * (2048 / b->cfg[kind].threads);
-    return std::max(1, std::min(nch, cap));
+    return std::max(1, b->cnt[kind][m]);
 }
 
 // launches of one stage for the kinds selected in `mask` (bit per work-list kind)
@@ -539,7 +543,7 @@ grmhd_status grmhd_batch_create(grmhd_ctx* const* ctxs, int n, void* scratch, si
     b->wait_limit_s = 1.0;
     b->persist_blocks = 0;
     b->nsm = ctx_nsm(ctxs[0]);
-    for (int k = 0; k < WL_KINDS; k++) b->cfg[k] = kCands[1];
+    for (int k = 0; k < WL_KINDS; k++) b->cfg[k] = kCands[0];
     for (int p = 0; p < n; p++) {
         fill_desc(b, p, 0.0);
         if (ctx_any_fixed(ctxs[p])) b->fixed_probs.push_back(p);
@@ -619,7 +623,7 @@ grmhd_status grmhd_batch_autotune(grmhd_batch* b, int reps, grmhd_stream_t strea
     for (int kind = 0; kind < WL_KINDS && res == GRMHD_OK; kind++) {
         if (!b->cnt[kind][0] && !b->cnt[kind][1]) continue;
         float best = 1e30f;
-        int bi = 1;
+        int bi = 0;
         for (int ci = 0; ci < kNCand; ci++) {
             b->cfg[kind] = kCands[ci];
             if ((res = build_lists(b, st)) != GRMHD_OK) break;

@@ -288,6 +288,7 @@ ImpArgs imp_args(grmhd_ctx* c, CP8 qb, CP3 bf, double a_dt, P8 prim, P3 R, P3 qE
     a.xi = c->xi;
     a.p32 = p32;
     a.nfail = c->nfail;
+    a.stage_qE = 0;
     for (int v = 0; v < 3; v++) a.hs[v] = a.hd[v] = nullptr;
     return a;
 }
@@ -1118,6 +1119,18 @@ void ctx_stage_args(grmhd_ctx* c, int i, double dt, ImpArgs* ia, UpdateArgs* a)
     }
     a->cwL = dt * c->tab.wt[i];
     a->cwR = dt * c->tab.w[i];
+    const double mh = -0.5 * c->g.idx[0];
+    for (int r = 0; r < S; r++) a->cLS[r] = a->cL[r] * mh;
+    a->cwLS = a->cwL * mh;
+    // FP64 with a metric: the implicit solve leaves q_E for the update's Gauss law, in the
+    // arrays of the ideal-limit EMF's transport velocities, which the resistive one does not use
+    if (!c->mixed && !c->glm && !c->ideal && (c->psi || c->alp)) {
+        ia->stage_qE = 1;
+        for (int d = 0; d < c->grid.ndim; d++) {
+            ia->qE_out.p[d] = c->vblk[d][0];
+            a->qE[d] = c->vblk[d][0];
+        }
+    }
     for (int v = 0; v < 3; v++) a->R[v] = c->R[v];
     for (int v = 0; v < 8; v++) a->qn[v] = c->q[v];
     for (int v = 0; v < 3; v++) a->qn[8 + v] = c->bf[v];

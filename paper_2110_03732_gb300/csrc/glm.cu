@@ -69,8 +69,10 @@ __device__ __forceinline__ void glm_update_item(const Dims& g, const GlmUpdateAr
     interior_coords(g, t, c);
     const long long o = lin(g, c[0], c[1], c[2]);
     double Lc[12];
+    cell_sources<M, true>(g, a.prim, a.qB, nullptr, psi, alp, c, o, Lc);
 #pragma unroll
-    for (int v = 0; v < 12; v++) Lc[v] = 0.0;
+    for (int v = 0; v < 12; v++)
+        if (v == 0 || v >= 8 || (!M && v < 5)) Lc[v] = 0.0;
 #pragma unroll
     for (int d = 0; d < 3; d++) {
         if (!g.act[d]) continue;
@@ -82,7 +84,6 @@ __device__ __forceinline__ void glm_update_item(const Dims& g, const GlmUpdateAr
             Lc[v] -= (Fv[o1] - Fv[o]) * hidx;
         }
     }
-    cell_sources<true>(g, a.prim, a.qB, psi, alp, c, o, Lc);
     const double ps = psi ? psi[o] : 1.0;
     const double al = alp ? alp[o] : 1.0;
     const double p2 = ps * ps;

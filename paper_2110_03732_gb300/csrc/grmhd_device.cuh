@@ -57,6 +57,7 @@ struct Dims {
     int n[3], ng[3], N[3], bc[3], act[3];
     long long st[3];       // strides of x, y, z
     double idx[3];         // 1/dx (0 where inactive)
+    double rdx[3];         // dx[0] / dx[d] (0 where inactive)
     double gh;             // Gamma_hat_1 = Gamma/(Gamma - 1)
     double igh;            // 1/Gamma_hat_1
     long long ncell;       // padded cells
@@ -84,6 +85,7 @@ inline void set_divisors(Dims& g)
     }
     for (int d = 0; d < 3; d++) {
         set_march(g, d, 1);
+        g.rdx[d] = g.act[d] ? g.idx[d] / g.idx[0] : 0.0;   // (direction 0 is always active)
         const double h = 0.5 * g.idx[d];
         g.hix[d][0] = (float)h;
         g.hix[d][1] = (float)(h - (double)g.hix[d][0]);

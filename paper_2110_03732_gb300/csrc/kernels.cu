@@ -35,13 +35,13 @@ thread_local bool launch_overlap = false;
 // update: cell-centred L (flux divergence + non-stiff sources) and face L_B (CT)
 // ---------------------------------------------------------------------------
 
-// The FP32-flux instances are held to 32 registers (16 blocks per SM, 300-570 B of
-// spills): the 513^2 items of a 512^2 stage then fit one wave instead of 1.5 and the
-// 128^3 star's mixed update ran 454 -> 421 us per launch (512^2: 42.8 -> 41.7 us).  The
-// FP64 instances keep the compiler's choice (64-78 registers): bound by the FP64 pipe,
-// they only lost from more blocks.
+// Register bounds, us per launch.  The FP32-flux instances take 32 registers (16 blocks per
+// SM; one variable at a time, 90-240 B of spills): 512^2 40.0 against 46.4 at 8 to 12 blocks,
+// 96^3 star 166 against 199-214 (42 and 181 with all eight divergences held at once).  FP64:
+// seven blocks flat (512^2 55.7; 56.5 unbounded, 58.2 at eight), ten with a metric (128^3
+// 748; 778 at twelve, 760 at eight; 903 before the sources were collected).
 template <bool M, bool F32>
-__global__ void __launch_bounds__(128, F32 ? 16 : 0) k_update(Dims g, UpdateArgs a)
+__global__ void __launch_bounds__(128, F32 ? 16 : (M ? 10 : 7)) k_update(Dims g, UpdateArgs a)
 {
     grid_dep_sync();
     long long tot = 1;

@@ -32,7 +32,8 @@ struct ImpArgs {
     float ighf, ighl, xif;  // 1/Gamma_hat as a double-word ighf + ighl, and FP32 xi
     P8 prim;                // in: Newton start; out: stage primitives
     P3 R;                   // stiff rates (or NULL)
-    P3 qE_out;              // solved q_E (or NULL)
+    P3 qE_out;              // solved q_E (or NULL entries)
+    int stage_qE;           // qE_out is the stage's own scratch (ctx_stage_args), not a caller's q
     int kmax;
     double tol, rho_atm, p_atm;
     float tolf;             // tol in FP32 (for the double-word corrections)
@@ -80,6 +81,8 @@ struct UpdateArgs {
     double At[4][4], A[4][4], wt[4], w[4];
     double cL[4], cR[4];    // dt At[k][stage], dt A[k][stage]: this stage's terms in base k
     double cwL, cwR;        // dt wt[stage], dt w[stage]: its terms in the final combination
+    double cLS[4], cwLS;    // cL[k] and cwL times -1 / (2 dx_0) (out_scaled)
+    const double* qE[3];    // solved q_E of the stage's interior cells (FP64 with a metric), or NULL
     const double* F[3][8];  // twice the face fluxes per active direction (float arrays when f32)
     int f32;                // the fluxes are FP32 (the mixed-precision flux kernels)
     const double* Eh[3];    // edge EMFs
