@@ -991,7 +991,9 @@ grmhd_status grmhd_clean_divb(grmhd_ctx* c, int cycles, void* scratch, size_t sc
     if (mg_plan(c->g, &plan) != 0) return grmhd_clean_scratch_bytes(&c->grid, &scratch_bytes);
     if (scratch_bytes < mg_scratch_bytes(plan))
         return fail(GRMHD_ERR_SCRATCH, "scratch smaller than grmhd_clean_scratch_bytes");
-    cudaError_t e = mg_clean(c->g, plan, (double*)scratch, c->bf, c->glm, cycles, c->nsm, (cudaStream_t)stream,
+    const OverlapScope ov(c->overlap);
+    // (two flux arrays serve as work space: no flux is kept from one stage to the next)
+    cudaError_t e = mg_clean(c->g, plan, (double*)scratch, c->F[0][0], c->F[0][1], c->bf, c->glm, cycles, c->nsm, (cudaStream_t)stream,
                              &c->launches);
     if (e != cudaSuccess) return cuda_fail(e, "multigrid kernels");
     return GRMHD_OK;

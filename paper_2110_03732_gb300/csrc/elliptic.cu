@@ -23,6 +23,7 @@
 
 #include "elliptic.h"
 #include "grmhd_device.cuh"
+#include "launch.cuh"
 
 namespace grmhd {
 
@@ -36,7 +37,7 @@ __device__ __forceinline__ long long mg_nb(const MgLevel& L, const int* bc, int 
     c[d] += s;
     if (c[d] < 0 || c[d] >= L.n[d]) {
         if (bc[d] != BC_PERIODIC) return -1;
-        c[d] = (c[d] + L.n[d]) % L.n[d];
+        c[d] += c[d] < 0 ? L.n[d] : -L.n[d];
     }
     return c[0] + (long long)L.n[0] * (c[1] + (long long)L.n[1] * c[2]);
 }
@@ -46,14 +47,15 @@ struct MgArgs {
     int act[3];
 };
 
-// cell (i, j, k) of level item t (levels hold fewer than 2^31 cells: mg_plan)
+// cell (i, j, k) of level item t (levels hold fewer than 2^31 cells: mg_plan); a division
+// by a run-time value would issue its conversions on the FP64 pipe
 __device__ __forceinline__ void mg_coords(const MgLevel& L, long long t, int& i, int& j, int& k)
 {
-    const int u = (int)t;
-    const int r = u / L.n[0];
-    i = u - r * L.n[0];
-    j = r % L.n[1];
-    k = r / L.n[1];
+    int c[3];
+    box_coords(t, L.f0, L.f1, c);
+    i = c[0];
+    j = c[1];
+    k = c[2];
 }
 
 // (L Phi)_c split as sum_nb Phi_nb / h^2 - diag Phi_c; returns the neighbour sum, the
@@ -100,12 +102,12 @@ __device__ __forceinline__ long long mg_half_items(const MgLevel& L)
 // diagonal reciprocal is the level's; a boundary cell (fewer neighbours) divides.
 __device__ __forceinline__ void mg_smooth_cell(const MgLevel& L, const MgArgs& m, int color, long long t)
 {
-    const int h0 = (L.n[0] + 1) >> 1;
-    const int u = (int)t, row = u / h0;
-    const int j = row % L.n[1], k = row / L.n[1];
-    const int i = 2 * (u - row * h0) + ((color + j + k) & 1);
+    int x[3];
+    box_coords(t, L.fh, L.f1, x);
+    const int j = x[1], k = x[2];
+    const int i = 2 * x[0] + ((color + j + k) & 1);
     if (i >= L.n[0]) return;
-    const int c = i + L.n[0] * row;
+    const int c = i + L.n[0] * (j + L.n[1] * k);
     double nbsum, diag;
     int miss;
     mg_stencil(L, m, L.phi, i, j, k, nbsum, diag, miss);
@@ -115,6 +117,7 @@ __device__ __forceinline__ void mg_smooth_cell(const MgLevel& L, const MgArgs& m
 
 __global__ void __launch_bounds__(256) k_mg_smooth(MgLevel L, MgArgs m, int color)
 {
+    grid_dep_sync();
     const long long items = mg_half_items(L);
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < items;
          t += (long long)gridDim.x * blockDim.x)
@@ -146,6 +149,7 @@ __device__ __forceinline__ void mg_restrict_cell(const MgLevel& F, const MgLevel
 
 __global__ void __launch_bounds__(256) k_mg_restrict(MgLevel F, MgLevel C, MgArgs m)
 {
+    grid_dep_sync();
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < C.cells;
          t += (long long)gridDim.x * blockDim.x)
         mg_restrict_cell(F, C, m, t);
@@ -177,7 +181,7 @@ __device__ __forceinline__ void mg_prolong_cell(const MgLevel& F, const MgLevel&
                         q[d] = P[d] + off[d] * S[d];
                         w *= off[d] ? 0.25 : 0.75;
                         if (q[d] < 0 || q[d] >= C.n[d]) {
-                            if (m.bc[d] == BC_PERIODIC) q[d] = (q[d] + C.n[d]) % C.n[d];
+                            if (m.bc[d] == BC_PERIODIC) q[d] += q[d] < 0 ? C.n[d] : -C.n[d];
                             else q[d] = P[d];
                         }
                     }
@@ -189,6 +193,7 @@ __device__ __forceinline__ void mg_prolong_cell(const MgLevel& F, const MgLevel&
 
 __global__ void __launch_bounds__(256) k_mg_prolong(MgLevel F, MgLevel C, MgArgs m)
 {
+    grid_dep_sync();
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < F.cells;
          t += (long long)gridDim.x * blockDim.x)
         mg_prolong_cell(F, C, m, t);
@@ -213,31 +218,52 @@ __device__ __forceinline__ double mg_block_sum(double v, double* sh)
     return sh[32];
 }
 
+// the block sum where one warp holds every value: five shuffles, no barrier
+template <bool W>
+__device__ __forceinline__ double mg_sum(double v, double* sh)
+{
+    if (!W) return mg_block_sum(v, sh);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+template <bool W>
+__device__ __forceinline__ void mg_sync()
+{
+    if (W) __syncwarp();
+    else __syncthreads();
+}
+
 // coarsest level: conjugate gradients on -lap (symmetric positive semi-definite) with
 // a mean-free right-hand side, in one block.  r, p and q are scratch vectors of the
 // level's size; iterations end at ||r|| <= 1e-15 ||b|| or after max_it.
-__device__ __forceinline__ void mg_cg_block(const MgLevel& L, const MgArgs& m, double* __restrict__ res,
-                                            double* __restrict__ p, double* __restrict__ q, int max_it, double* sh)
+//
+// W: by the first warp alone (the callers' other warps wait), for a level of so few cells
+// that the block barriers of the sums would cost more than the arithmetic. 
+template <bool W>
+__device__ __forceinline__ void mg_cg_run(const MgLevel& L, const MgArgs& m, double* __restrict__ res,
+                                          double* __restrict__ p, double* __restrict__ q, int max_it, double* sh)
 {
-    const long long n = L.cells;
+    const int n = (int)L.cells, nt = W ? 32 : (int)blockDim.x;
     // b = -(rhs - mean rhs); x = 0, r = b, p = r
     double s = 0.0;
-    for (long long t = threadIdx.x; t < n; t += blockDim.x) s += L.rhs[t];
-    const double mean = mg_block_sum(s, sh) / (double)n;
+    for (int t = threadIdx.x; t < n; t += nt) s += L.rhs[t];
+    const double mean = mg_sum<W>(s, sh) / (double)n;
     double rr = 0.0;
-    for (long long t = threadIdx.x; t < n; t += blockDim.x) {
+    for (int t = threadIdx.x; t < n; t += nt) {
         const double b = -(L.rhs[t] - mean);
         res[t] = b;
         p[t] = b;
         L.phi[t] = 0.0;
         rr += b * b;
     }
-    rr = mg_block_sum(rr, sh);
+    rr = mg_sum<W>(rr, sh);
     const double stop = 1e-30 * rr;
     for (int it = 0; it < max_it && rr > stop && rr > 0.0; it++) {
         // q = -lap p
         double pq = 0.0;
-        for (long long t = threadIdx.x; t < n; t += blockDim.x) {
+        for (int t = threadIdx.x; t < n; t += nt) {
             int i, j, k;
             mg_coords(L, t, i, j, k);
             double nbsum, diag;
@@ -247,23 +273,34 @@ __device__ __forceinline__ void mg_cg_block(const MgLevel& L, const MgArgs& m, d
             q[t] = v;
             pq += p[t] * v;
         }
-        pq = mg_block_sum(pq, sh);
+        pq = mg_sum<W>(pq, sh);
         if (!(pq > 0.0)) break;
         const double alpha = rr / pq;
         double rn = 0.0;
-        for (long long t = threadIdx.x; t < n; t += blockDim.x) {
+        for (int t = threadIdx.x; t < n; t += nt) {
             L.phi[t] += alpha * p[t];
             const double r = res[t] - alpha * q[t];
             res[t] = r;
             rn += r * r;
         }
-        rn = mg_block_sum(rn, sh);
+        rn = mg_sum<W>(rn, sh);
         const double beta = rn / rr;
         rr = rn;
-        for (long long t = threadIdx.x; t < n; t += blockDim.x) p[t] = res[t] + beta * p[t];
-        __syncthreads();
+        for (int t = threadIdx.x; t < n; t += nt) p[t] = res[t] + beta * p[t];
+        mg_sync<W>();
     }
-    __syncthreads();
+    mg_sync<W>();
+}
+
+__device__ __forceinline__ void mg_cg_block(const MgLevel& L, const MgArgs& m, double* __restrict__ res,
+                                            double* __restrict__ p, double* __restrict__ q, int max_it, double* sh)
+{
+    if (L.cells <= 64) {
+        if (threadIdx.x < 32) mg_cg_run<true>(L, m, res, p, q, max_it, sh);
+        __syncthreads();
+    } else {
+        mg_cg_run<false>(L, m, res, p, q, max_it, sh);
+    }
 }
 
 // the levels first..nlev-1 (each at most kMgBlockCells cells) of one V-cycle in a
@@ -296,6 +333,7 @@ __device__ __forceinline__ MgLevel tail_level(const MgTail& T, int l, double* sm
 __global__ void __launch_bounds__(1024) k_mg_tail(MgTail T, MgArgs m, double* __restrict__ res,
                                                    double* __restrict__ p, double* __restrict__ q, int max_it)
 {
+    grid_dep_sync();
     extern __shared__ double tail_sm[];
     __shared__ double sh[33];
     if (T.smem) {
@@ -341,10 +379,173 @@ __global__ void __launch_bounds__(1024) k_mg_tail(MgTail T, MgArgs m, double* __
     }
 }
 
+// ---------------------------------------------------------------------------
+// 2-D levels: the four half sweeps of a leg and its transfer in one launch
+// ---------------------------------------------------------------------------
+
+// A block owns a T x T tile and holds it with a halo of H cells in shared memory.  Half sweep
+// s updates the cells up to H - 1 - s from the tile (those of its colour), so that each
+// needs only cells the half sweep before has updated: every cell gets the value the
+// grid-wide half sweeps give it (to rounding), the halo's being computed by each block that
+// needs them.  The legs write to the level's other Phi array, since a block's halo is
+// another block's tile.  A leg took five launches of 4-9 us, each a few hundred cycles of
+// work; the redundant halo cells cost less than those.
+template <int T, int H>
+struct MgTile {
+    static constexpr int R = T + 2 * H;
+    double phi[R][R + 1], rs[R][R + 1];   // Phi and rhs / diagonal of the full stencil
+};
+
+// level coordinate of region coordinate r of a tile at o: wrapped, or -1 outside a
+// non-periodic extent (o - H + 2n >= 0: fused levels have n >= 4)
+__device__ __forceinline__ int mg_wrap(int x, int n, const FastDiv& f, bool periodic)
+{
+    if (x >= 0 && x < n) return x;
+    if (!periodic) return -1;
+    const unsigned u = (unsigned)(x + 2 * n);
+    return (int)(u - fdiv(u, f) * (unsigned)n);
+}
+
+// Phi of the region cell (rx, ry) by one Gauss-Seidel update; x, y its level coordinates.
+// A cell beside a non-periodic boundary has fewer neighbours and divides.
+template <int T, int H>
+__device__ __forceinline__ double mg_tile_update(const MgLevel& L, const MgArgs& m, const MgTile<T, H>& S, int rx,
+                                                 int ry, int x, int y)
+{
+    const bool bx = m.bc[0] != BC_PERIODIC && (x == 0 || x == L.n[0] - 1);
+    const bool by = m.bc[1] != BC_PERIODIC && (y == 0 || y == L.n[1] - 1);
+    const double l = S.phi[ry][rx - 1], r = S.phi[ry][rx + 1], d = S.phi[ry - 1][rx], u = S.phi[ry + 1][rx];
+    if (!bx && !by) return fma(l + r, L.cx[0], fma(d + u, L.cx[1], -S.rs[ry][rx]));
+    double nb = 0.0, diag = 0.0;
+    if (!(bx && x == 0)) { nb += l * L.ih2[0]; diag += L.ih2[0]; }
+    if (!(bx && x == L.n[0] - 1)) { nb += r * L.ih2[0]; diag += L.ih2[0]; }
+    if (!(by && y == 0)) { nb += d * L.ih2[1]; diag += L.ih2[1]; }
+    if (!(by && y == L.n[1] - 1)) { nb += u * L.ih2[1]; diag += L.ih2[1]; }
+    return diag > 0.0 ? (nb - S.rs[ry][rx] * L.dfull) / diag : S.phi[ry][rx];
+}
+
+template <int T, int H>
+__device__ __forceinline__ void mg_tile_sweeps(const MgLevel& L, const MgArgs& m, MgTile<T, H>& S, int ox, int oy)
+{
+    const bool px = m.bc[0] == BC_PERIODIC, py = m.bc[1] == BC_PERIODIC;
+#pragma unroll
+    for (int s = 0; s < 4; s++) {
+        constexpr int e0 = H - 1;
+        const int e = e0 - s, w = T + 2 * e, hw = w / 2;   // T + 2e is even
+        __syncthreads();
+        for (int t = threadIdx.x; t < w * hw; t += blockDim.x) {
+            const int row = t / hw, ry = H - e + row;
+            const int y = oy + ry - H;
+            // colour (x + y) & 1 of the unwrapped coordinates: extents are even
+            const int rx0 = H - e, x0 = ox + rx0 - H;
+            const int rx = rx0 + 2 * (t - row * hw) + ((x0 + y + s) & 1);
+            const int gx = mg_wrap(ox + rx - H, L.n[0], L.f0, px), gy = mg_wrap(y, L.n[1], L.f1, py);
+            if (gx < 0 || gy < 0) continue;
+            S.phi[ry][rx] = mg_tile_update<T, H>(L, m, S, rx, ry, gx, gy);
+        }
+    }
+    __syncthreads();
+}
+
+// down leg: four half sweeps from L.phi (zero: from 0), Phi to L.alt, the residual averaged
+// to the coarse right-hand side, and the coarse Phi set to zero
+template <int T>
+__global__ void __launch_bounds__(256) k_mg_down2(MgLevel L, MgLevel C, MgArgs m, int zero)
+{
+    constexpr int H = 5;
+    __shared__ MgTile<T, H> S;
+    grid_dep_sync();
+    const int ox = blockIdx.x * T, oy = blockIdx.y * T;
+    constexpr int R = MgTile<T, H>::R;
+    for (int t = threadIdx.x; t < R * R; t += blockDim.x) {
+        const int ry = t / R, rx = t - ry * R;
+        const int gx = mg_wrap(ox + rx - H, L.n[0], L.f0, m.bc[0] == BC_PERIODIC);
+        const int gy = mg_wrap(oy + ry - H, L.n[1], L.f1, m.bc[1] == BC_PERIODIC);
+        const bool in = gx >= 0 && gy >= 0;
+        const long long c = in ? gx + (long long)L.n[0] * gy : 0;
+        S.phi[ry][rx] = in && !zero ? L.phi[c] : 0.0;
+        S.rs[ry][rx] = in ? L.rhs[c] * L.idiag : 0.0;
+    }
+    mg_tile_sweeps<T, H>(L, m, S, ox, oy);
+    for (int t = threadIdx.x; t < T * T; t += blockDim.x) {
+        const int ty = t / T, tx = t - ty * T;
+        if (ox + tx < L.n[0] && oy + ty < L.n[1])
+            L.alt[ox + tx + (long long)L.n[0] * (oy + ty)] = S.phi[ty + H][tx + H];
+    }
+    for (int t = threadIdx.x; t < T * T / 4; t += blockDim.x) {
+        const int cy = t / (T / 2), cx = t - cy * (T / 2);
+        const int X = ox / 2 + cx, Y = oy / 2 + cy;
+        if (X >= C.n[0] || Y >= C.n[1]) continue;
+        double sum = 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int rx = 2 * cx + (k & 1) + H, ry = 2 * cy + (k >> 1) + H;
+            const int x = ox + rx - H, y = oy + ry - H;
+            const bool edge = (m.bc[0] != BC_PERIODIC && (x == 0 || x == L.n[0] - 1)) ||
+                              (m.bc[1] != BC_PERIODIC && (y == 0 || y == L.n[1] - 1));
+            const double f = S.phi[ry][rx];
+            if (!edge) {
+                // residual / dfull = rs - (neighbour sum) idiag + Phi
+                sum += (S.rs[ry][rx] + f) - fma(S.phi[ry][rx - 1] + S.phi[ry][rx + 1], L.cx[0],
+                                                (S.phi[ry - 1][rx] + S.phi[ry + 1][rx]) * L.cx[1]);
+            } else {
+                double r = S.rs[ry][rx] * L.dfull;
+                if (m.bc[0] == BC_PERIODIC || x > 0) r -= (S.phi[ry][rx - 1] - f) * L.ih2[0];
+                if (m.bc[0] == BC_PERIODIC || x < L.n[0] - 1) r -= (S.phi[ry][rx + 1] - f) * L.ih2[0];
+                if (m.bc[1] == BC_PERIODIC || y > 0) r -= (S.phi[ry - 1][rx] - f) * L.ih2[1];
+                if (m.bc[1] == BC_PERIODIC || y < L.n[1] - 1) r -= (S.phi[ry + 1][rx] - f) * L.ih2[1];
+                sum += r * L.idiag;
+            }
+        }
+        const long long c = X + (long long)C.n[0] * Y;
+        C.rhs[c] = sum * (0.25 * L.dfull);
+        C.phi[c] = 0.0;
+    }
+}
+
+// up leg: the coarse correction interpolated onto L.alt (as mg_prolong_cell), then four half
+// sweeps; Phi to L.phi
+template <int T>
+__global__ void __launch_bounds__(256) k_mg_up2(MgLevel L, MgLevel C, MgArgs m)
+{
+    constexpr int H = 4;
+    __shared__ MgTile<T, H> S;
+    grid_dep_sync();
+    const int ox = blockIdx.x * T, oy = blockIdx.y * T;
+    constexpr int R = MgTile<T, H>::R;
+    const bool px = m.bc[0] == BC_PERIODIC, py = m.bc[1] == BC_PERIODIC;
+    for (int t = threadIdx.x; t < R * R; t += blockDim.x) {
+        const int ry = t / R, rx = t - ry * R;
+        const int gx = mg_wrap(ox + rx - H, L.n[0], L.f0, px), gy = mg_wrap(oy + ry - H, L.n[1], L.f1, py);
+        double v = 0.0, rs = 0.0;
+        if (gx >= 0 && gy >= 0) {
+            const long long c = gx + (long long)L.n[0] * gy;
+            rs = L.rhs[c] * L.idiag;
+            const int X = gx >> 1, Y = gy >> 1;
+            int X1 = X + ((gx & 1) ? 1 : -1), Y1 = Y + ((gy & 1) ? 1 : -1);
+            if (X1 < 0 || X1 >= C.n[0]) X1 = px ? (X1 < 0 ? X1 + C.n[0] : X1 - C.n[0]) : X;
+            if (Y1 < 0 || Y1 >= C.n[1]) Y1 = py ? (Y1 < 0 ? Y1 + C.n[1] : Y1 - C.n[1]) : Y;
+            const long long r0 = (long long)C.n[0] * Y, r1 = (long long)C.n[0] * Y1;
+            const double a = fma(0.25, C.phi[X1 + r0], 0.75 * C.phi[X + r0]);
+            const double b = fma(0.25, C.phi[X1 + r1], 0.75 * C.phi[X + r1]);
+            v = fma(0.25, b, fma(0.75, a, L.alt[c]));
+        }
+        S.phi[ry][rx] = v;
+        S.rs[ry][rx] = rs;
+    }
+    mg_tile_sweeps<T, H>(L, m, S, ox, oy);
+    for (int t = threadIdx.x; t < T * T; t += blockDim.x) {
+        const int ty = t / T, tx = t - ty * T;
+        if (ox + tx < L.n[0] && oy + ty < L.n[1])
+            L.phi[ox + tx + (long long)L.n[0] * (oy + ty)] = S.phi[ty + H][tx + H];
+    }
+}
+
 // fine right-hand side: div q_B on the interior cells (faces or central), and block
 // partial sums for its mean
 __global__ void __launch_bounds__(256) k_mg_div(Dims g, CP3 bq, int cc, MgLevel L, MgArgs m, double* __restrict__ part)
 {
+    grid_dep_sync();
     __shared__ double sh[33];
     double s = 0.0;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < L.cells;
@@ -386,6 +587,7 @@ __global__ void __launch_bounds__(256) k_mg_div(Dims g, CP3 bq, int cc, MgLevel 
 __global__ void __launch_bounds__(256) k_mg_mean(const double* __restrict__ part, int nb, double* __restrict__ mean,
                                                  long long cells)
 {
+    grid_dep_sync();
     __shared__ double sh[33];
     double s = 0.0;
     for (int b = threadIdx.x; b < nb; b += blockDim.x) s += part[b];
@@ -395,6 +597,7 @@ __global__ void __launch_bounds__(256) k_mg_mean(const double* __restrict__ part
 
 __global__ void __launch_bounds__(256) k_mg_sub_mean(MgLevel L, const double* __restrict__ mean)
 {
+    grid_dep_sync();
     const double mu = *mean;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < L.cells;
          t += (long long)gridDim.x * blockDim.x)
@@ -405,6 +608,7 @@ __global__ void __launch_bounds__(256) k_mg_sub_mean(MgLevel L, const double* __
 // of a non-periodic direction is kept) or central (cell-centred)
 __global__ void __launch_bounds__(256) k_mg_correct(Dims g, P3 bq, int cc, MgLevel L, MgArgs m)
 {
+    grid_dep_sync();
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < L.cells;
          t += (long long)gridDim.x * blockDim.x) {
         int c[3];
@@ -467,6 +671,10 @@ int mg_plan(const Dims& g, MgPlan* plan)
                 L.dfull += L.ih2[d];
             }
         L.idiag = L.dfull > 0.0 ? 1.0 / L.dfull : 0.0;
+        for (int d = 0; d < 3; d++) L.cx[d] = L.ih2[d] * L.idiag;
+        L.f0 = make_fastdiv((unsigned)n[0]);
+        L.f1 = make_fastdiv((unsigned)n[1]);
+        L.fh = make_fastdiv((unsigned)((n[0] + 1) / 2));
         if (cells >= (1LL << 31)) return -3;
         L.cells = cells;
         L.offset = total;
@@ -492,8 +700,8 @@ size_t mg_scratch_bytes(const MgPlan& p)
     return sizeof(double) * (2 * (size_t)p.total + 3 * coarse + kMgParts + 1);
 }
 
-cudaError_t mg_clean(const Dims& g, const MgPlan& plan0, double* scratch, double* const* bq, bool cc, int cycles,
-                     int nsm, cudaStream_t st, long long* launches)
+cudaError_t mg_clean(const Dims& g, const MgPlan& plan0, double* scratch, double* alt0, double* alt1,
+                     double* const* bq, bool cc, int cycles, int nsm, cudaStream_t st, long long* launches)
 {
     long long nl = 0;
     MgPlan plan = plan0;
@@ -503,6 +711,7 @@ cudaError_t mg_clean(const Dims& g, const MgPlan& plan0, double* scratch, double
         MgLevel& L = plan.lev[l];
         L.phi = scratch + L.offset;
         L.rhs = scratch + T + L.offset;
+        L.alt = l == 0 ? alt0 : alt1 + (L.offset - plan.lev[0].cells);
     }
     double* cg_r = scratch + 2 * T;
     double* cg_p = cg_r + nc;
@@ -523,11 +732,11 @@ cudaError_t mg_clean(const Dims& g, const MgPlan& plan0, double* scratch, double
     }
     const int nb = (int)((F.cells + 255) / 256 < kMgParts ? (F.cells + 255) / 256 : kMgParts);
     nl++;
-    k_mg_div<<<nb, 256, 0, st>>>(g, cq, cc ? 1 : 0, F, m, part);
+    launch_k(k_mg_div, nb, 256, st, g, cq, cc ? 1 : 0, F, m, part);
     nl++;
-    k_mg_mean<<<1, 256, 0, st>>>(part, nb, mean, F.cells);
+    launch_k(k_mg_mean, 1, 256, st, (const double*)part, nb, mean, F.cells);
     nl++;
-    k_mg_sub_mean<<<mg_grid(F.cells, nsm), 256, 0, st>>>(F, mean);
+    launch_k(k_mg_sub_mean, mg_grid(F.cells, nsm), 256, st, F, (const double*)mean);
     const int cg_it = (int)(2 * nc + 20);
     // levels of at most kMgBlockCells cells run inside one block (k_mg_tail)
     MgTail tail;
@@ -544,39 +753,57 @@ cudaError_t mg_clean(const Dims& g, const MgPlan& plan0, double* scratch, double
     const size_t tail_bytes = sizeof(double) * (size_t)(soff + 3 * nc);
     tail.smem = tail_bytes <= kMgTailSmem ? 1 : 0;
     const size_t tail_dyn = tail.smem ? tail_bytes : 0;
+    // 2-D levels: a leg per launch, in tiles of 32 cells a side where those fill the SMs, else 16
+    const bool tiled = g.act[0] && g.act[1] && !g.act[2];
+    auto tile_side = [&](const MgLevel& L) { return L.cells >= (long long)nsm * 1024 ? 32 : 16; };
     for (int cyc = 0; cyc < cycles; cyc++) {
         for (int l = 0; l < tail.first; l++) {
             const MgLevel& L = plan.lev[l];
+            if (tiled) {
+                nl++;
+                const int T = tile_side(L);
+                const dim3 gr((L.n[0] + T - 1) / T, (L.n[1] + T - 1) / T);
+                launch_dyn(T == 32 ? k_mg_down2<32> : k_mg_down2<16>, gr, 256, 0, st, L, plan.lev[l + 1], m,
+                           (cyc == 0 || l > 0) ? 1 : 0);
+                continue;
+            }
             const int bs = mg_grid(half_items(L), nsm);
             for (int s = 0; s < 2; s++) {
                 nl++;
-                k_mg_smooth<<<bs, 256, 0, st>>>(L, m, 0);
+                launch_k(k_mg_smooth, bs, 256, st, L, m, 0);
                 nl++;
-                k_mg_smooth<<<bs, 256, 0, st>>>(L, m, 1);
+                launch_k(k_mg_smooth, bs, 256, st, L, m, 1);
             }
             nl++;
-            k_mg_restrict<<<mg_grid(plan.lev[l + 1].cells, nsm), 256, 0, st>>>(L, plan.lev[l + 1], m);
+            launch_k(k_mg_restrict, mg_grid(plan.lev[l + 1].cells, nsm), 256, st, L, plan.lev[l + 1], m);
         }
         // the small levels and the coarsest solve (from zero); with a single level this
         // is the whole solve, and further cycles would repeat it
         nl++;
-        k_mg_tail<<<1, 1024, tail_dyn, st>>>(tail, m, cg_r, cg_p, cg_q, cg_it);
+        launch_dyn(k_mg_tail, dim3(1), 1024, tail_dyn, st, tail, m, cg_r, cg_p, cg_q, cg_it);
         if (plan.nlev == 1) break;
         for (int l = tail.first - 1; l >= 0; l--) {
             const MgLevel& L = plan.lev[l];
+            if (tiled) {
+                nl++;
+                const int T = tile_side(L);
+                const dim3 gr((L.n[0] + T - 1) / T, (L.n[1] + T - 1) / T);
+                launch_dyn(T == 32 ? k_mg_up2<32> : k_mg_up2<16>, gr, 256, 0, st, L, plan.lev[l + 1], m);
+                continue;
+            }
             const int b = mg_grid(L.cells, nsm), bs = mg_grid(half_items(L), nsm);
             nl++;
-            k_mg_prolong<<<b, 256, 0, st>>>(L, plan.lev[l + 1], m);
+            launch_k(k_mg_prolong, b, 256, st, L, plan.lev[l + 1], m);
             for (int s = 0; s < 2; s++) {
                 nl++;
-                k_mg_smooth<<<bs, 256, 0, st>>>(L, m, 0);
+                launch_k(k_mg_smooth, bs, 256, st, L, m, 0);
                 nl++;
-                k_mg_smooth<<<bs, 256, 0, st>>>(L, m, 1);
+                launch_k(k_mg_smooth, bs, 256, st, L, m, 1);
             }
         }
     }
     nl++;
-    k_mg_correct<<<mg_grid(F.cells, nsm), 256, 0, st>>>(g, pq, cc ? 1 : 0, F, m);
+    launch_k(k_mg_correct, mg_grid(F.cells, nsm), 256, st, g, pq, cc ? 1 : 0, F, m);
     if (launches) *launches += nl;
     return cudaGetLastError();
 }

@@ -22,10 +22,13 @@ struct MgLevel {
     double ih2[3];        // 1/h^2 per active direction, 0 otherwise
     double dfull, idiag;  // diagonal of the full (2 ndim + 1)-point stencil (summed in
                           // the device's order) and its reciprocal
+    double cx[3];         // ih2 * idiag
+    FastDiv f0, f1, fh;   // divisions by n[0], n[1] and ceil(n[0] / 2)
     long long cells;
-    long long offset;     // of this level's arrays in the phi / rhs blocks
+    long long offset;     // of this level's arrays in the phi / rhs / alt blocks
     double* phi;
     double* rhs;
+    double* alt;          // Phi between the legs of a cycle (2-D levels run by k_mg_down2 / k_mg_up2)
 };
 
 struct MgPlan {
@@ -40,7 +43,9 @@ int mg_plan(const Dims& g, MgPlan* plan);
 size_t mg_scratch_bytes(const MgPlan& plan);
 // clean the three q_B arrays bq in place (staggered faces, or cell-centred if cc) with
 // `cycles` V-cycles; scratch of mg_scratch_bytes(plan) bytes (8-byte aligned)
-cudaError_t mg_clean(const Dims& g, const MgPlan& plan, double* scratch, double* const* bq, bool cc, int cycles,
-                     int nsm, cudaStream_t st, long long* launches);
+// alt0, alt1: two more arrays of the padded grid's cells (2-D: the second Phi of the finest
+// level and of the others)
+cudaError_t mg_clean(const Dims& g, const MgPlan& plan, double* scratch, double* alt0, double* alt1,
+                     double* const* bq, bool cc, int cycles, int nsm, cudaStream_t st, long long* launches);
 
 }  // namespace grmhd

@@ -28,22 +28,28 @@ __device__ __forceinline__ void grid_dep_sync()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// k<<<grid, block, 0, st>>>(args...), with the programmatic attribute when
+// k<<<grid, block, smem, st>>>(args...), with the programmatic attribute when
 // launch_overlap is set.  k must open with grid_dep_sync().
 template <typename... P, typename... A>
-inline cudaError_t launch_k(void (*k)(P...), int grid, int block, cudaStream_t st, A&&... args)
+inline cudaError_t launch_dyn(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A&&... args)
 {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = launch_overlap ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k, std::forward<A>(args)...);
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_k(void (*k)(P...), int grid, int block, cudaStream_t st, A&&... args)
+{
+    return launch_dyn(k, dim3((unsigned)grid), block, 0, st, std::forward<A>(args)...);
 }
 
 // blocks of `threads` for `work` items, at most 16 per SM (the kernels stride)
