@@ -133,8 +133,7 @@ template <int C, bool M, typename T>
 __device__ __forceinline__ void emf_any_item(const ProbStage& ps, long long t)
 {
     if (ps.g.act[(C + 1) % 3] && ps.g.act[(C + 2) % 3]) {
-        if constexpr (sizeof(T) == 8) emf64_item<M, false>(ps.g, C, ps.p64.p, ps.bfs.p, ps.psi, ps.alp, ps.Eh64[C], t);
-        else emf_march_item<C, M, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp, ps.Eh64[C], t);
+        emf_line_item<M, T, false>(ps.g, C, prim_of<T>(ps).p, ps.bfs.p, ps.psi, ps.alp, ps.Eh64[C], t);
     } else {
         emf_item<C, M, T>(ps.g, prim_of<T>(ps), ps.bfs, ps.psi, ps.alp, ps.Eh64[C], t);
     }

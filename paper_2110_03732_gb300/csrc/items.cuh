@@ -326,10 +326,10 @@ __device__ __forceinline__ T uct_edge(T hLL, T hLR, T hRL, T hRR, T ca, T cb, T 
     return scale_pow2<T, -2>(hLL + hLR + hRL + hRR) + (T(0.5) * ca) * (qBbR - qBbL) - (T(0.5) * cb) * (qBaR - qBaL);
 }
 
-// HLL flux at the D-face with padded coordinates c (between the cells of linear
-// indices rm = c - e_D and r0 = c) from the reconstructed states: prL / prR the 8
-// primitives (coordinate u^i and E^i), BL / BR the coordinate B with the two transverse
-// components set (the normal one is the face's own).  Writes twice the flux at r0.  prL,
+// HLL flux at the D-face of linear index r0 (that of the cell above it) from the
+// reconstructed states: prL / prR the 8 primitives (coordinate u^i and E^i), BL / BR the
+// coordinate B with the two transverse components set; Bn the face's own normal q_B, psf and
+// alf psi and alpha at the face (psi: whether there is one).  Writes twice the flux at r0.  prL,
 // prR, BL, BR are overwritten.  FP32 (mixed precision).
 //
 // Eh (flat metric only, else NULL): Eh[C] set for an edge direction C != D whose
@@ -339,20 +339,16 @@ __device__ __forceinline__ T uct_edge(T hLL, T hLR, T hRL, T hRR, T ca, T cb, T 
 // computes from the same MC or PPM values (to round-off: the edge formula here is
 // reduced for the coinciding states).
 template <int D, bool M>
-__device__ __forceinline__ void face_flux32(const Dims& g, const CP3& bf, const double* psi_in, const double* alp_in,
-                                            const int* c, long long rm, long long r0, float* prL, float* prR,
-                                            float* BL, float* BR, const FluxOut<float>& F, double* const* Eh)
+__device__ __forceinline__ void face_flux32(const Dims& g, float Bn, bool psi, float psf, float alf, long long r0,
+                                            float* prL, float* prR, float* BL, float* BR, const FluxOut<float>& F,
+                                            double* const* Eh)
 {
     using T = float;
-    const double* __restrict__ psi = M ? psi_in : nullptr;
-    const double* __restrict__ alp = M ? alp_in : nullptr;
     constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
-    const T psf = psi ? mean2<T>(psi[rm], psi[r0]) : T(1);
-    const T alf = alp ? mean2<T>(alp[rm], alp[r0]) : T(1);
     const T pf2 = psf * psf, ipf2 = psi ? rcp_t(pf2) : T(1);
     // orthonormal-frame states at the face: u_hat = psi^2 u, E_hat = psi^2 E,
     // B_hat = psi^2 B (normal: q_B / psi^4)
-    BL[D] = BR[D] = (T)bf.p[D][face_at(g, D, c)] * (ipf2 * ipf2);
+    BL[D] = BR[D] = Bn * (ipf2 * ipf2);
     if (!M && Eh) {
         // C = D + 1: A = D + 2 (inactive), B = D; C = D + 2: A = D, B = D + 1 (inactive)
         // uct_edge with the inactive side's two states equal: the four-state mean is
@@ -542,55 +538,81 @@ __device__ __forceinline__ void flux32_item(const Dims& g, const PrimIn<float>& 
     using T = float;
     using Rec = LineRec<T, P>;
     const double* __restrict__ psi = M ? psi_in : nullptr;
+    const double* __restrict__ alp = M ? alp_in : nullptr;
     constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
     constexpr int NV = 10;   // 8 primitives and the two transverse B
     int c[3], f0, f1;
     march_coords<D>(g, t, c, f0, f1);
+    // the line's cells lie at line + m st[D] (the other coordinates are interior)
+    const long long sd = g.st[D];
+    long long line = 0;
+#pragma unroll
+    for (int d = 0; d < 3; d++)
+        if (d != D) line += c[d] * g.st[d];
     // the 10 reconstructed values of the cell at padded coordinate m along D (PPM's
-    // stencil reaches a third ghost: ext_cell maps it)
-    auto load = [&](int m, T* x) {
-        int cs[3] = {c[0], c[1], c[2]};
-        cs[D] = P ? ext_cell(g, D, m) : m;
-        const long long mi = cell_at(g, cs);
+    // stencil reaches a third ghost: ext_cell maps it); ps: psi there, in FP32
+    auto load = [&](int m, T* x, T& ps) {
+        const int mx = P ? ext_cell(g, D, m) : m;
+        const long long mi = chk(g, line + map_cell(g, D, mx) * sd);
 #pragma unroll
         for (int v = 0; v < 8; v++) x[v] = prim.p[v][mi];
         T ip6 = T(1);
+        ps = T(1);
         if (psi) {
-            const T ps = met_t<T>(psi[lin(g, cs[0], cs[1], cs[2])]), p2 = ps * ps;
+            ps = met_t<T>(psi[chk(g, line + mx * sd)]);
+            const T p2 = ps * ps;
             ip6 = rcp_t(p2 * p2 * p2);
         }
         x[8] = prim.p[8 + T1][mi] * ip6;
         x[9] = prim.p[8 + T2][mi] * ip6;
     };
     Rec rec[NV];
+    // the metric of the cells f - 1 and f beside the face, converted once per cell: psA, psB
+    // (psN: the AHEAD newer cells, the newest last) and alA
+    T psA = T(1), psB = T(1), psN[Rec::AHEAD], alA = T(1);
     {
-        T w[2][NV];
+        T w[2][NV], pw[2];
 #pragma unroll
-        for (int k = 0; k < 2; k++) load(f0 - Rec::WARM + Rec::AHEAD - 2 + k, w[k]);
+        for (int k = 0; k < 2; k++) load(f0 - Rec::WARM + Rec::AHEAD - 2 + k, w[k], pw[k]);
 #pragma unroll
         for (int v = 0; v < NV; v++) {
             rec[v].push(w[0][v]);
             rec[v].push(w[1][v]);
         }
+        if (P) {
+            psN[0] = pw[0];
+            psN[Rec::AHEAD - 1] = pw[1];
+        } else {
+            psB = pw[0];
+            psN[0] = pw[1];
+        }
     }
-    int cm[3] = {c[0], c[1], c[2]};
-    cm[D] = f0 - 1;
-    long long rm = lin(g, cm[0], cm[1], cm[2]);
+    if (alp) alA = met_t<T>(alp[chk(g, line + (f0 - 1) * sd)]);
     for (int f = f0 - Rec::WARM; f < f1; f++) {
-        T x[NV];
-        load(f + Rec::AHEAD, x);
+        T x[NV], psx;
+        load(f + Rec::AHEAD, x, psx);
         T prL[NV], prR[NV];
         line_step<NV>(rec, x, prL, prR);
+        psA = psB;
+        psB = psN[0];
+        if (P) psN[0] = psN[Rec::AHEAD - 1];
+        psN[Rec::AHEAD - 1] = psx;
         if (f < f0) continue;
         T BL[3], BR[3];
         BL[T1] = prL[8];
         BL[T2] = prL[9];
         BR[T1] = prR[8];
         BR[T2] = prR[9];
-        c[D] = f;
-        const long long r0 = lin(g, c[0], c[1], c[2]);
-        face_flux32<D, M>(g, bf, psi_in, alp_in, c, rm, r0, prL, prR, BL, BR, F, Eh);
-        rm = r0;
+        const long long r0 = chk(g, line + f * sd);
+        T psf = T(1), alf = T(1);
+        if (psi) psf = T(0.5) * (psA + psB);
+        if (alp) {
+            const T alB = met_t<T>(alp[r0]);
+            alf = T(0.5) * (alA + alB);
+            alA = alB;
+        }
+        face_flux32<D, M>(g, (T)bf.p[D][chk(g, line + map_face(g, D, f) * sd)], psi != nullptr, psf, alf, r0, prL, prR,
+                          BL, BR, F, Eh);
     }
 }
 
@@ -1022,107 +1044,6 @@ __device__ __forceinline__ void emf_item(const Dims& g, const PrimIn<T>& prim, c
     Eh[i0] = to_f64(uct_edge<T>(hLL, hLR, hRL, hRR, ca, cb, qBbL, qBbR, qBaL, qBaR));
 }
 
-// The same EMFs for K consecutive C-edges along B per thread (MC, or PPM when P; A and
-// B both active): the A-direction reconstruction of E_C on each row of cells along B,
-// and q_B^A, are marched along B with LineRec (one new row per edge instead of four or
-// six), so each edge computes one A-row, three one-cell B steps and its own q_B^B
-// reconstruction.  The results are bitwise those of emf_item.  Items: chunks of K edges
-// along B, x-fastest over the other two directions (the chunks run along x when B = 0).
-template <int C, bool M, typename T, bool P = false>
-__device__ __forceinline__ void emf_march_item(const Dims& g, const PrimIn<T>& prim, const CP3& bf,
-                                               const double* psi_in, const double* alp_in, double* __restrict__ Eh,
-                                               long long t)
-{
-    using Rec = LineRec<T, P>;
-    constexpr int NS = P ? 6 : 4, OFF = P ? 3 : 2;
-    const double* __restrict__ psi = M ? psi_in : nullptr;
-    const double* __restrict__ alp = M ? alp_in : nullptr;
-    constexpr int A = (C + 1) % 3, B = (C + 2) % 3;
-    const T* __restrict__ Ec = prim.p[5 + C];
-    const int K = g.mk[B];
-    // x-fastest box: the chunks along B, n[C] edges along C, n[A] + 1 along A
-    int c[3], idx[3];
-    box_coords(t, B == 0 ? g.dq[0] : (C == 0 ? g.dv[0] : g.dvp[0]),
-               B == 1 ? g.dq[1] : (C == 1 ? g.dv[1] : g.dvp[1]), idx);
-#pragma unroll
-    for (int d = 0; d < 3; d++) c[d] = g.ng[d] + (d == B ? 0 : idx[d]);
-    const int f0 = g.ng[B] + idx[B] * K;
-    const int f1 = min(f0 + K, g.ng[B] + g.n[B] + 1);
-    // a face state along A from the NS values v (cells or faces c[A]-OFF..)
-    auto recA = [&](const T* v, T& L, T& R) {
-        if (P) ppm_face<T>(v, L, R);
-        else mc_face<T>(v[0], v[1], v[2], v[NS - 1], L, R);
-    };
-    // row m along B: covariant E_C = psi^4 E^C reconstructed along A to the A-face c[A],
-    // and q_B^A at that A-face
-    auto row = [&](int m, T* x) {
-        const int mb = P ? ext_cell(g, B, m) : m;
-        T v[NS];
-#pragma unroll
-        for (int sa = 0; sa < NS; sa++) {
-            int cs[3] = {c[0], c[1], c[2]};
-            cs[B] = mb;
-            cs[A] = P ? ext_cell(g, A, c[A] + sa - OFF) : c[A] + sa - OFF;
-            const T ps = psi ? met_t<T>(psi[lin(g, cs[0], cs[1], cs[2])]) : T(1);
-            const T p2 = ps * ps;
-            v[sa] = p2 * p2 * Ec[cell_at(g, cs)];
-        }
-        recA(v, x[0], x[1]);
-        int cs[3] = {c[0], c[1], c[2]};
-        cs[B] = mb;
-        x[2] = (T)bf.p[A][face_at(g, A, cs)];
-    };
-    Rec rec[3];
-#pragma unroll
-    for (int v = 0; v < 3; v++) {
-        rec[v].push(T(0));
-        rec[v].push(T(0));
-    }
-    for (int f = f0 - Rec::WARM - 2; f < f1; f++) {
-        T x3[3];
-        row(f + Rec::AHEAD, x3);
-        if (f < f0 - Rec::WARM) {
-#pragma unroll
-            for (int v = 0; v < 3; v++) rec[v].push(x3[v]);
-            continue;
-        }
-        T L[3], R[3];
-        line_step<3>(rec, x3, L, R);
-        if (f < f0) continue;
-        c[B] = f;
-        // q_B^B (B-faces) along A
-        T qBbL, qBbR;
-        {
-            T v[NS];
-#pragma unroll
-            for (int sa = 0; sa < NS; sa++) {
-                int cs[3] = {c[0], c[1], c[2]};
-                cs[A] = P ? ext_cell(g, A, c[A] + sa - OFF) : c[A] + sa - OFF;
-                v[sa] = (T)bf.p[B][face_at(g, B, cs)];
-            }
-            recA(v, qBbL, qBbR);
-        }
-        const long long i0 = lin(g, c[0], c[1], c[2]);
-        const long long sA = g.st[A], sB = g.st[B];
-        T ale = T(1), ca = T(1), cb = T(1);
-        if (alp || psi) {
-            T sum = alp ? met_t<T>(alp[i0]) : T(1);
-            sum += alp ? met_t<T>(alp[chk(g, i0 - sA)]) : T(1);
-            sum += alp ? met_t<T>(alp[chk(g, i0 - sB)]) : T(1);
-            sum += alp ? met_t<T>(alp[chk(g, i0 - sA - sB)]) : T(1);
-            ale = sum * T(0.25);
-            T cab[2];
-            edge_speeds<T>(g, psi, alp, i0, true, true, sA, sB, cab);
-            ca = cab[0];
-            cb = cab[1];
-        }
-        // EXY[X][Y]: X the A side (the row's L / R), Y the B side (L = this edge's
-        // lower-B state)
-        Eh[i0] = to_f64(uct_edge<T>(ale * L[0], ale * R[0], ale * L[1], ale * R[1], ca, cb, qBbL, qBbR, L[2],
-                                     R[2]));
-    }
-}
-
 // The metric of a C-edge among the four cells c00, cA (one below along A), cB and cAB: the
 // lapse there (their mean) and half the larger of the two A-face speeds alpha / psi^2 and
 // of the two B-face ones (alpha and psi at a face: the means of its two cells).  The larger
@@ -1163,19 +1084,24 @@ __device__ __forceinline__ void edge_metric64(const double* __restrict__ psi, co
     hb = num[1] * (den[0] * r);
 }
 
-// emf_march_item in FP64 with the edge direction C a run-time value (the launch's tasks
-// share one code) and the line's offsets formed once: the same reconstructions and sums.
-template <bool M, bool P>
-__device__ __forceinline__ void emf64_item(const Dims& g, int C, const double* const* prim, const double* const* bf,
-                                           const double* psi_in, const double* alp_in, double* __restrict__ Eh,
-                                           long long t)
+// The EMFs of K consecutive C-edges along B per thread (MC, or PPM when P; A and B both
+// active): the A-direction reconstruction of E_C on each row of cells along B, and q_B^A,
+// are marched along B with LineRec (one new row per edge instead of four or six), so each
+// edge computes one A-row, three one-cell B steps and its own q_B^B reconstruction, with the
+// sums of emf_item (in FP32 bitwise).  Items: chunks of K edges along B, x-fastest over the
+// other two directions (the chunks run along x when B = 0).  C is a run-time value (the tasks
+// of a launch share one code) and the line's offsets are formed once.
+template <bool M, typename T, bool P>
+__device__ __forceinline__ void emf_line_item(const Dims& g, int C, const T* const* prim, const double* const* bf,
+                                              const double* psi_in, const double* alp_in, double* __restrict__ Eh,
+                                              long long t)
 {
-    using Rec = LineRec<double, P>;
+    using Rec = LineRec<T, P>;
     constexpr int NS = P ? 6 : 4, OFF = P ? 3 : 2;
     const double* __restrict__ psi = M ? psi_in : nullptr;
     const double* __restrict__ alp = M ? alp_in : nullptr;
     const int A = C == 2 ? 0 : C + 1, B = C == 0 ? 2 : C - 1;
-    const double* __restrict__ Ec = prim[5 + C];
+    const T* __restrict__ Ec = prim[5 + C];
     const double* __restrict__ qA = bf[A];
     const double* __restrict__ qB = bf[B];
     // x-fastest box: the chunks along B, n[C] edges along C, n[A] + 1 along A
@@ -1195,62 +1121,85 @@ __device__ __forceinline__ void emf64_item(const Dims& g, int C, const double* c
         pa[k] = line + m * sA;
     }
     const long long fa = line + map_face(g, A, cA) * sA;
-    auto recA = [&](const double* v, double& L, double& R) {
-        if (P) ppm_face<double>(v, L, R);
-        else mc_face<double>(v[0], v[1], v[2], v[NS - 1], L, R);
+    auto recA = [&](const T* v, T& L, T& R) {
+        if (P) ppm_face<T>(v, L, R);
+        else mc_face<T>(v[0], v[1], v[2], v[NS - 1], L, R);
     };
     Rec rec[3];
 #pragma unroll
     for (int v = 0; v < 3; v++) {
-        rec[v].push(0.0);
-        rec[v].push(0.0);
+        rec[v].push(T(0));
+        rec[v].push(T(0));
     }
     for (int f = f0 - Rec::WARM - 2; f < f1; f++) {
         // row f + AHEAD along B: covariant E_C = psi^4 E^C reconstructed along A to the
         // A-face, and q_B^A at that A-face
         const int mb = P ? ext_cell(g, B, f + Rec::AHEAD) : f + Rec::AHEAD;
         const long long rb = map_cell(g, B, mb) * sB;
-        double x3[3];
+        T x3[3];
         {
-            double v[NS];
+            T v[NS];
+            if constexpr (sizeof(T) == 8) {
 #pragma unroll
-            for (int k = 0; k < NS; k++) {
-                v[k] = Ec[chk(g, ia[k] + rb)];
-                if (psi) {
-                    const double ps = psi[chk(g, pa[k] + mb * sB)], p2 = ps * ps;
-                    v[k] *= p2 * p2;
+                for (int k = 0; k < NS; k++) {
+                    v[k] = Ec[chk(g, ia[k] + rb)];
+                    if (psi) {
+                        const T ps = psi[chk(g, pa[k] + mb * sB)], p2 = ps * ps;
+                        v[k] *= p2 * p2;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < NS; k++) {
+                    const T ps = psi ? met_t<T>(psi[chk(g, pa[k] + mb * sB)]) : T(1);
+                    const T p2 = ps * ps;
+                    v[k] = p2 * p2 * Ec[chk(g, ia[k] + rb)];
                 }
             }
             recA(v, x3[0], x3[1]);
         }
-        x3[2] = qA[chk(g, fa + rb)];
+        x3[2] = (T)qA[chk(g, fa + rb)];
         if (f < f0 - Rec::WARM) {
 #pragma unroll
             for (int v = 0; v < 3; v++) rec[v].push(x3[v]);
             continue;
         }
-        double L[3], R[3];
+        T L[3], R[3];
         line_step<3>(rec, x3, L, R);
         if (f < f0) continue;
         // q_B^B (B-faces) along A
-        double qL, qR;
+        T qL, qR;
         {
             const long long jb = map_face(g, B, f) * sB;
-            double v[NS];
+            T v[NS];
 #pragma unroll
-            for (int k = 0; k < NS; k++) v[k] = qB[chk(g, ia[k] + jb)];
+            for (int k = 0; k < NS; k++) v[k] = (T)qB[chk(g, ia[k] + jb)];
             recA(v, qL, qR);
         }
         const long long i0 = chk(g, line + cA * sA + f * sB);
-        // uct_edge: the mean of the four states times the edge's lapse, and half the larger
-        // face speed of each direction times the jump of q_B
-        const double mean = scale_pow2<double, -2>((L[0] + R[0]) + (L[1] + R[1]));
-        if (alp || psi) {
-            double ale, ha, hb;
-            edge_metric64(psi, alp, i0, chk(g, i0 - sA), chk(g, i0 - sB), chk(g, i0 - sA - sB), ale, ha, hb);
-            Eh[i0] = fma(-hb, R[2] - L[2], fma(ha, qR - qL, ale * mean));
+        if constexpr (sizeof(T) == 8) {
+            // uct_edge: the mean of the four states times the edge's lapse, and half the larger
+            // face speed of each direction times the jump of q_B
+            const double mean = scale_pow2<double, -2>((L[0] + R[0]) + (L[1] + R[1]));
+            if (alp || psi) {
+                double ale, ha, hb;
+                edge_metric64(psi, alp, i0, chk(g, i0 - sA), chk(g, i0 - sB), chk(g, i0 - sA - sB), ale, ha, hb);
+                Eh[i0] = fma(-hb, R[2] - L[2], fma(ha, qR - qL, ale * mean));
+            } else {
+                Eh[i0] = fma(-0.5, R[2] - L[2], fma(0.5, qR - qL, mean));
+            }
         } else {
-            Eh[i0] = fma(-0.5, R[2] - L[2], fma(0.5, qR - qL, mean));
+            T ale = T(1), cab[2] = {T(1), T(1)};
+            if (alp || psi) {
+                T sum = alp ? met_t<T>(alp[i0]) : T(1);
+                sum += alp ? met_t<T>(alp[chk(g, i0 - sA)]) : T(1);
+                sum += alp ? met_t<T>(alp[chk(g, i0 - sB)]) : T(1);
+                sum += alp ? met_t<T>(alp[chk(g, i0 - sA - sB)]) : T(1);
+                ale = sum * T(0.25);
+                edge_speeds<T>(g, psi, alp, i0, true, true, sA, sB, cab);
+            }
+            Eh[i0] = to_f64(uct_edge<T>(ale * L[0], ale * R[0], ale * L[1], ale * R[1], cab[0], cab[1], qL, qR, L[2],
+                                        R[2]));
         }
     }
 }

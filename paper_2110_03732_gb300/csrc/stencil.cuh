@@ -65,16 +65,13 @@ __device__ __forceinline__ void stencil_emf_single(const Dims& g, const EmfArgs<
     for (long long t = t0; t < tot; t += nt) emf_item<C, M, T, P>(g, a.prim, a.bf, a.psi, a.alp, a.Eh, t);
 }
 
-// marched edges of direction c (FP32: c = C)
-template <int C, bool M, typename T, bool P>
+// marched edges of direction c
+template <bool M, typename T, bool P>
 __device__ __forceinline__ void stencil_emf_march(const Dims& g, int c, const EmfArgs<T>& a, long long t0, long long nt)
 {
     const int A = c == 2 ? 0 : c + 1, B = c == 0 ? 2 : c - 1;
     const long long tot = (long long)g.dq[B].d * g.n[c] * (g.n[A] + 1);
-    for (long long t = t0; t < tot; t += nt) {
-        if constexpr (sizeof(T) == 8) emf64_item<M, P>(g, c, a.prim.p, a.bf.p, a.psi, a.alp, a.Eh, t);
-        else emf_march_item<C, M, T, P>(g, a.prim, a.bf, a.psi, a.alp, a.Eh, t);
-    }
+    for (long long t = t0; t < tot; t += nt) emf_line_item<M, T, P>(g, c, a.prim.p, a.bf.p, a.psi, a.alp, a.Eh, t);
 }
 
 // The FP32 PPM instance is held to 96 registers (five blocks per SM, 160 B of spills):
@@ -91,29 +88,20 @@ __global__ void __launch_bounds__(stencil_threads<T, P>(), sizeof(T) == 8 ? 4 : 
         if (b >= L.b0[i]) s = i;   // empty tasks have b0[i] == b0[i + 1]
     const long long nt = (long long)(L.b0[s + 1] - L.b0[s]) * blockDim.x;
     const long long t0 = (long long)(b - L.b0[s]) * blockDim.x + threadIdx.x;
+    // the FP64 fluxes and the marched edges take the direction as a run-time value: one code
     if constexpr (sizeof(T) == 8) {
-        // FP64: the direction is a run-time value, one code for the fluxes and one for the
-        // marched edges
         if (s < 3) {
             stencil_flux<0, M, T, P>(L.g[s], s, L.fa[s], t0, nt, sm);
             return;
         }
-        if (L.emarch[s - 3]) {
-            stencil_emf_march<0, M, T, P>(L.g[s], s - 3, L.ea[s - 3], t0, nt);
-            return;
-        }
+    }
+    if (s >= 3 && L.emarch[s - 3]) {
+        stencil_emf_march<M, T, P>(L.g[s], s - 3, L.ea[s - 3], t0, nt);
+        return;
     }
     switch (s) {
 #define GRMHD_STENCIL_EMF(C)                                                                       \
-    case 3 + C:                                                                                    \
-        if constexpr (sizeof(T) == 4) {                                                            \
-            if (L.emarch[C]) {                                                                     \
-                stencil_emf_march<C, M, T, P>(L.g[3 + C], C, L.ea[C], t0, nt);                     \
-                break;                                                                             \
-            }                                                                                      \
-        }                                                                                          \
-        stencil_emf_single<C, M, T, P>(L.g[3 + C], L.ea[C], t0, nt);                          \
-        break;
+    case 3 + C: stencil_emf_single<C, M, T, P>(L.g[3 + C], L.ea[C], t0, nt); break;
 #define GRMHD_STENCIL_FLUX(D)                                                                      \
     case D:                                                                                        \
         if constexpr (sizeof(T) == 4) stencil_flux<D, M, T, P>(L.g[D], D, L.fa[D], t0, nt, sm);    \
