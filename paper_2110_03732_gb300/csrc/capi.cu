@@ -412,7 +412,7 @@ grmhd_status explicit_part(grmhd_ctx* c, CP8 prim, CP3 bfs, UpdateArgs& a, cudaS
     return GRMHD_OK;
 }
 
-// GLM (Sec. 3.1): fluxes of the 12 cell-centred variables per direction, then the
+// GLM (Sec. 3.1): fluxes of the 12 cell-centred variables (one launch), then the
 // update; qB / qphi are the stage's cell fields
 grmhd_status explicit_part_glm(grmhd_ctx* c, CP8 prim, CP3 qB, const double* qphi, GlmUpdateArgs& a,
                                cudaStream_t st)
@@ -425,15 +425,13 @@ grmhd_status explicit_part_glm(grmhd_ctx* c, CP8 prim, CP3 qB, const double* qph
     fa.qphi = qphi;
     fa.psi = c->psi;
     fa.alp = c->alp;
-    for (int d = 0; d < 3; d++) {
-        if (!g.act[d]) continue;
-        for (int v = 0; v < 12; v++) fa.F[v] = c->F[d][v];
-        const int tk = tbegin(c, KIND_FLUX, st);
-        e = launch_glm_flux(g, d, fa, c->nsm, st, c->ppm);
-        tend(c, tk, st);
-        c->launches++;
-        if (e != cudaSuccess) return cuda_fail(e, "GLM flux kernel");
-    }
+    for (int d = 0; d < 3; d++)
+        for (int v = 0; v < 12; v++) fa.F[d][v] = g.act[d] ? c->F[d][v] : nullptr;
+    const int tf = tbegin(c, KIND_FLUX, st);
+    e = launch_glm_flux(g, fa, c->nsm, st, c->ppm);
+    tend(c, tf, st);
+    c->launches++;
+    if (e != cudaSuccess) return cuda_fail(e, "GLM flux kernel");
     for (int d = 0; d < 3; d++)
         for (int v = 0; v < 12; v++) a.F[d][v] = g.act[d] ? c->F[d][v] : nullptr;
     for (int v = 0; v < 8; v++) a.prim[v] = prim.p[v];

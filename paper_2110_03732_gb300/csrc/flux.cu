@@ -8,7 +8,7 @@
 
 namespace grmhd {
 
-// MC (or PPM) fluxes, K consecutive D-faces per thread (flux_march_item)
+// MC (or PPM) fluxes, K consecutive D-faces per thread (flux64_item)
 template <int D, bool M, bool P = false>
 __global__ void __launch_bounds__(Flux64<P, false>::NT, 4) k_flux_march(Dims g, FluxArgs<double> a)
 {

@@ -660,12 +660,14 @@ __device__ __forceinline__ void hll_half64(const double* st, const double* Bt, d
 }
 
 // Threads per block of the kernels that run flux64_item, and the shared doubles it takes
-// (SL per thread and quantity: MC a, b, lo, hi; PPM a0, a1, s0, ip, lo, hi)
+// (SL per thread and quantity: MC a, b, lo, hi; PPM a0, a1, s0, ip, lo, hi).  us per stencil
+// launch by threads per block and least blocks per SM: MC 512^2 128 x 4 116.5, 128 x 5 117.1,
+// 96 x 5 121.1, 64 x 8 117.6; PPM 301^2 96 x 4 159.1, 64 x 6 155.1, 64 x 7 166.5, 32 x 14 167.9.
 template <bool P, bool CC>
 struct Flux64 {
     static constexpr int NV = CC ? 12 : 10;        // 8 primitives, B_t1, B_t2 (CC: B_n, B_t1, B_t2, Phi)
     static constexpr int SL = P ? 6 : 4;
-    static constexpr int NT = !P ? 128 : (CC ? 64 : 96);
+    static constexpr int NT = P ? 64 : 128;
     static constexpr int SM = NV * SL * NT;        // at most 48 KB
 };
 

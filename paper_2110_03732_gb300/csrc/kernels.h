@@ -60,7 +60,7 @@ struct FluxArgs {
     FluxOut<T> F;           // twice the face fluxes (FP32 values in mixed precision)
     double* vbar[2];        // ideal-limit EMF: transverse transport velocities (or NULL)
     double* Eh[3];          // edge EMFs written by the flux kernel (flat 1-D / 2-D grids,
-                            // see face_flux), NULL for those the EMF kernels compute
+                            // see flux64_item), NULL for those the EMF kernels compute
 };
 
 template <typename T>
@@ -143,7 +143,7 @@ struct GlmFluxArgs {
     const double* qphi;     // stage q_Phi
     const double* psi;
     const double* alp;
-    double* F[12];          // twice the face fluxes of the 12 variables along the launch direction
+    double* F[3][12];       // twice the face fluxes of the 12 variables per active direction
 };
 
 struct GlmUpdateArgs {
@@ -167,7 +167,8 @@ struct GlmUpdateArgs {
 };
 
 cudaError_t launch_implicit_cc(const Dims& g, const ImpArgs& a, int nsm, cudaStream_t st);
-cudaError_t launch_glm_flux(const Dims& g, int d, const GlmFluxArgs& a, int nsm, cudaStream_t st, bool ppm = false);
+// the fluxes of every active direction in one launch
+cudaError_t launch_glm_flux(const Dims& g, const GlmFluxArgs& a, int nsm, cudaStream_t st, bool ppm = false);
 cudaError_t launch_glm_update(const Dims& g, const GlmUpdateArgs& a, int nsm, cudaStream_t st);
 cudaError_t launch_curlA_cc(const Dims& g, CP3 A, P3 qB, int nsm, cudaStream_t st);
 cudaError_t launch_prim2con_cc(const Dims& g, CP8 prim, CP3 qB, const double* psi, const double* phi, double* qphi,

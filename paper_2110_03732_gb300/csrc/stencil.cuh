@@ -77,7 +77,7 @@ __device__ __forceinline__ void stencil_emf_march(const Dims& g, int c, const Em
 // The FP32 PPM instance is held to 96 registers (five blocks per SM, 160 B of spills):
 // at its natural 128 it ran 2 % slower.  The others keep the compiler's choice.
 template <bool M, typename T, bool P>
-__global__ void __launch_bounds__(stencil_threads<T, P>(), sizeof(T) == 8 ? 4 : (P ? 5 : 0)) k_stencil(StencilTasks<T> L)
+__global__ void __launch_bounds__(stencil_threads<T, P>(), sizeof(T) == 8 ? (P ? 6 : 4) : (P ? 5 : 0)) k_stencil(StencilTasks<T> L)
 {
     __shared__ double sm[sizeof(T) == 8 ? Flux64<P, false>::SM : 1];
     grid_dep_sync();
