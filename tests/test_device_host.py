@@ -1,0 +1,112 @@
+"""The per-cell device code (csrc/*.cuh) compiled as plain C++ (device_on_host.h) and run on
+the CPU at inputs where a rule inside it can go wrong."""
+import shutil
+import subprocess
+from pathlib import Path
+
+import pytest
+
+ROOT = Path(__file__).resolve().parents[1]
+CUDA = Path(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc").resolve().parents[1] / "include"
+
+pytestmark = pytest.mark.skipif(shutil.which("g++") is None or not (CUDA / "cuda_runtime.h").exists(),
+                                reason="no g++ or CUDA headers")
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    """The rows (lists of floats) through the program `src`, a list of floats back for each."""
+    built = {}
+
+    def call(src, rows):
+        if src not in built:
+            d = tmp_path_factory.mktemp("device")
+            (d / "t.cpp").write_text('#include "device_on_host.h"\n' + src)
+            inc = [ROOT / "tests", CUDA, ROOT / "paper_2110_03732_gb300" / "csrc", ROOT / "include"]
+            subprocess.run(["g++", "-O1", "-std=c++17", "-ffp-contract=off", *(f"-I{i}" for i in inc), str(d / "t.cpp"),
+                            "-o", str(d / "t")], check=True)
+            built[src] = d / "t"
+        text = "\n".join(" ".join(float(x).hex() for x in r) for r in rows) + "\n"
+        out = subprocess.run([str(built[src])], input=text, capture_output=True, text=True, check=True).stdout
+        return [[float.fromhex(x) for x in ln.split()] for ln in out.splitlines()]
+
+    return call
+
+
+# one cell of a flat 1-D grid of four: the conserved variables of a state, and the solve from
+# another start
+IMPLICIT = r"""
+#include <cstdio>
+#include "grmhd_device.cuh"
+#include "items.cuh"
+using namespace grmhd;
+int main() {
+    double s, r, a_dt;   // density scale, field scale (r r = s), a_ii dt
+    while (std::scanf("%la %la %la", &s, &r, &a_dt) == 3) {
+        Dims g = {};
+        g.n[0] = 4; g.n[1] = g.n[2] = 1;
+        g.ng[0] = 2; g.N[0] = 8; g.N[1] = g.N[2] = 1;
+        g.act[0] = 1;
+        g.st[0] = 1; g.st[1] = g.st[2] = 8;
+        g.idx[0] = 4.0;
+        g.gh = 4.0; g.igh = 0.25;
+        g.ncell = 8;
+        set_divisors(g);
+        const double rho = 1.3 * s, p = 0.7 * s, u[3] = {0.4, -0.6, 0.3}, E[3] = {0.5 * r, 0.2 * r, -0.3 * r},
+                     B[3] = {0.6 * r, -0.8 * r, 0.5 * r};
+        const double W = std::sqrt(1 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]), hW = (rho + 4.0 * p) * W;
+        double q[8], U = 0;
+        for (int i = 0; i < 3; i++) U += 0.5 * (E[i] * E[i] + B[i] * B[i]);
+        q[0] = rho * W;
+        for (int i = 0; i < 3; i++) {
+            const int j = (i + 1) % 3, k = (i + 2) % 3;
+            q[1 + i] = hW * u[i] + E[j] * B[k] - E[k] * B[j];
+            q[5 + i] = E[i];
+        }
+        q[4] = hW * W - p + U - q[0];
+        double A[30][8];
+        ImpArgs a = {};
+        for (int v = 0; v < 8; v++) {
+            for (int c = 0; c < 8; c++) A[v][c] = q[v];
+            a.qb.p[v] = A[v];
+            a.prim.p[v] = A[11 + v];
+        }
+        const double start[8] = {s, 0.1, 0.1, 0.1, s, 0, 0, 0};
+        for (int c = 0; c < 8; c++)
+            for (int v = 0; v < 8; v++) A[11 + v][c] = start[v];
+        for (int d = 0; d < 3; d++) {
+            for (int c = 0; c < 8; c++) A[8 + d][c] = B[d];
+            a.bf.p[d] = A[8 + d];
+            a.R.p[d] = A[19 + d];
+            a.qE_out.p[d] = A[22 + d];
+        }
+        unsigned long long nfail = 0;
+        a.eta_u = 0.01;
+        a.a_dt = a_dt;
+        a.ia_dt = a_dt > 0 ? 1 / a_dt : 0;
+        a.stiff = a_dt > 0;
+        a.ighf = 0.25f;
+        a.kmax = 50;
+        a.tol = 1e-13;
+        a.tolf = 1e-13f;
+        a.nfail = &nfail;
+        implicit_item<false, false, false>(g, a, 1);
+        std::printf("%a %a %a %a %a %a\n", (double)nfail, A[11][3] / s, A[12][3], A[13][3], A[14][3], A[15][3] / s);
+    }
+}
+"""
+
+
+@pytest.mark.parametrize("a_dt", [0.0, 0.05])
+def test_implicit_solve_at_any_scale(run, a_dt):
+    """The equations of the implicit solve do not change when densities are multiplied by s and
+    fields by its root: the velocity and the scaled density and pressure stay the same, also where
+    the momentum leaves the range of FP32.  1e-11: the 1e-13 of the residual test on both
+    sides, and the condition of this state (below 10)."""
+    r = [2.0 ** k for k in (0, -40, 40, 64, 70, 100)]
+    rows = run(IMPLICIT, [[x * x, x, a_dt] for x in r])
+    assert all(row[0] == 0 for row in rows)
+    if a_dt == 0.0:   # E held fixed: the state itself is the root
+        assert rows[0][1:] == pytest.approx([1.3, 0.4, -0.6, 0.3, 0.7], rel=1e-11)
+    for row in rows[1:]:
+        assert row[1:] == pytest.approx(rows[0][1:], rel=1e-11)
