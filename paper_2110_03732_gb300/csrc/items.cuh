@@ -1390,7 +1390,9 @@ __device__ __forceinline__ void cell_sources(const Dims& g, const double* const*
         // s_S and s_tau for beta = 0, K_ij = 0 (Sec. 2.1) in the orthonormal frame:
         //   s_S_i = psi^6 [-(tau + D) d_i alpha + 2 alpha (d_i psi / psi)(rho h W^2 v^2 + 3p + U)]
         //   s_tau = -psi^4 S_hat_i d_i alpha
-        // with rho h W^2 v^2 + 3p + U = (tau + D) - rho h + 4p
+        // (the trace rho h W^2 v^2 + 3p + U is summed from its positive terms: as (tau + D) - rho h
+        // + 4p it would lose the digits of p / rho in a cold gas, where it is the whole source of
+        // a metric with psi alone)
         const double rho = prim[0][o], p = prim[4][o];
         const double ip4 = rcp_pos(p4);   // psi^-4; psi^-1 = psi^3 psi^-4
         double uh[3], Eh[3], Bh[3];
@@ -1403,7 +1405,7 @@ __device__ __forceinline__ void cell_sources(const Dims& g, const double* const*
         const double rhoh = fma(g.gh, p, rho), W = xw * iW, hW = rhoh * W;
         const double U2 = fma(Eh[0], Eh[0], fma(Eh[1], Eh[1], fma(Eh[2], Eh[2], fma(Bh[0], Bh[0], fma(Bh[1], Bh[1], Bh[2] * Bh[2])))));
         const double tauD = fma(hW, W, fma(0.5, U2, -p));   // tau + D
-        const double tr = fma(4.0, p, tauD - rhoh);
+        const double tr = fma(rhoh, p4 * u2, fma(3.0, p, 0.5 * U2));
         const double ktr = 2.0 * al * (ps * p2 * ip4) * tr;
         double s4 = 0.0;
 #pragma unroll

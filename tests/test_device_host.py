@@ -2,6 +2,7 @@
 the CPU at inputs where a rule inside it can go wrong."""
 import shutil
 import subprocess
+from fractions import Fraction as Fr
 from pathlib import Path
 
 import pytest
@@ -33,25 +34,33 @@ def run(tmp_path_factory):
     return call
 
 
-# one cell of a flat 1-D grid of four: the conserved variables of a state, and the solve from
-# another start
-IMPLICIT = r"""
+GRID = r"""
 #include <cstdio>
 #include "grmhd_device.cuh"
 #include "items.cuh"
 using namespace grmhd;
+// a 1-D grid of four cells
+Dims grid4()
+{
+    Dims g = {};
+    g.n[0] = 4; g.n[1] = g.n[2] = 1;
+    g.ng[0] = 2; g.N[0] = 8; g.N[1] = g.N[2] = 1;
+    g.act[0] = 1;
+    g.st[0] = 1; g.st[1] = g.st[2] = 8;
+    g.idx[0] = 4.0;
+    g.gh = 4.0; g.igh = 0.25;
+    g.ncell = 8;
+    set_divisors(g);
+    return g;
+}
+"""
+
+# the conserved variables of a state in a flat cell, and the solve from another start
+IMPLICIT = GRID + r"""
 int main() {
     double s, r, a_dt;   // density scale, field scale (r r = s), a_ii dt
     while (std::scanf("%la %la %la", &s, &r, &a_dt) == 3) {
-        Dims g = {};
-        g.n[0] = 4; g.n[1] = g.n[2] = 1;
-        g.ng[0] = 2; g.N[0] = 8; g.N[1] = g.N[2] = 1;
-        g.act[0] = 1;
-        g.st[0] = 1; g.st[1] = g.st[2] = 8;
-        g.idx[0] = 4.0;
-        g.gh = 4.0; g.igh = 0.25;
-        g.ncell = 8;
-        set_divisors(g);
+        const Dims g = grid4();
         const double rho = 1.3 * s, p = 0.7 * s, u[3] = {0.4, -0.6, 0.3}, E[3] = {0.5 * r, 0.2 * r, -0.3 * r},
                      B[3] = {0.6 * r, -0.8 * r, 0.5 * r};
         const double W = std::sqrt(1 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]), hW = (rho + 4.0 * p) * W;
@@ -110,3 +119,38 @@ def test_implicit_solve_at_any_scale(run, a_dt):
         assert rows[0][1:] == pytest.approx([1.3, 0.4, -0.6, 0.3, 0.7], rel=1e-11)
     for row in rows[1:]:
         assert row[1:] == pytest.approx(rows[0][1:], rel=1e-11)
+
+
+# the sources of a cell on a metric with psi alone
+SOURCES = GRID + r"""
+int main() {
+    double rho, p, f;   // density, pressure, size of u, E and B
+    while (std::scanf("%la %la %la", &rho, &p, &f) == 3) {
+        const Dims g = grid4();
+        double A[11][8], psi[8], src[8];
+        const double st[11] = {rho, f, -2 * f, f, p, 2 * f, f, -f, f, f, 2 * f};
+        const double *prim[8], *bf[3];
+        for (int c = 0; c < 8; c++) {
+            for (int v = 0; v < 11; v++) A[v][c] = st[v];
+            psi[c] = 1.0 + 0.125 * c;
+        }
+        for (int v = 0; v < 8; v++) prim[v] = A[v];
+        for (int d = 0; d < 3; d++) bf[d] = A[8 + d];
+        const int c[3] = {4, 0, 0};
+        cell_sources<true, false>(g, prim, bf, nullptr, psi, nullptr, c, 4, src);
+        std::printf("%a\n", src[1]);
+    }
+}
+"""
+
+
+def test_momentum_source_of_a_cold_gas(run):
+    """s_S = psi^6 2 alpha (d psi / psi) (rho h W^2 v^2 + 3 p + U) (Sec. 2.1) where the pressure and
+    the fields are far below the rest mass: a sum of positive terms, so 1e-14 (thirty roundings of
+    2^-53, and the reciprocal of psi^4 to an ulp or so) holds whatever their size."""
+    rows = [[rho, rho * 10.0 ** -k, m] for rho in (1.0, 1e-13) for k in (1, 5, 8, 11) for m in (0.0, 1e-9, 0.5)]
+    for (rho, p, f), (got,) in zip(rows, run(SOURCES, rows)):
+        rho, p, f, psi = Fr(rho), Fr(p), Fr(f), Fr(3, 2)
+        u2, U = psi ** 4 * 6 * f * f, (psi ** 4 * 6 * f * f + 6 * f * f / psi ** 8) / 2
+        want = psi ** 6 * 2 * (Fr(1, 4) * 2 / psi) * ((rho + 4 * p) * u2 + 3 * p + U)
+        assert abs(Fr(got) - want) <= want / 10 ** 14
