@@ -668,6 +668,14 @@ __device__ __forceinline__ double rcp_pos(double x)
     return fma(y, fma(e, e, e), y);
 }
 
+// the bounds of the two as high words: 1 + u^2 of a caller's velocity above 1.3e19 and W above
+// 8.5e37 take the library's forms
+constexpr unsigned kHi2p127 = 0x47e00000u, kHi2p126 = 0x47d00000u;
+
+// 1/sqrt(x) and 1/x for any x >= 1 (infinities and NaN as the library)
+__device__ __forceinline__ double rsqrt_wide(double x) { return mag_below_int(x, kHi2p127) ? rsqrt_ge1(x) : rsqrt(x); }
+__device__ __forceinline__ double rcp_wide(double x) { return mag_below_int(x, kHi2p126) ? rcp_pos(x) : 1.0 / x; }
+
 // 1/x for a positive x of moderate size in the stencil precision T (metric factors,
 // speed products): rcp_pos in FP64, the division in FP32
 __device__ __forceinline__ double rcp_t(double x) { return rcp_pos(x); }

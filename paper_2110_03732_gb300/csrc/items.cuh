@@ -643,6 +643,7 @@ __device__ __forceinline__ void hll_half64(const double* st, const double* Bt, d
     const double y = f2d_int(rsqrtf(d2f_int(x)));
     const double s = x * y, e = fma(-s, y, 1.0);
     W = fma(s, e * fma(0.375, e, 0.5), s);
+    if (!mag_below_int(x, kHi2p127)) W = x * rsqrt(x);   // the estimate has left the range of FP32
     const double h = fma(gh, p, rho), hW = h * W;
     const double e1 = SG > 0 ? Bt[1] + st[6] : Bt[1] - st[6];
     const double e2 = SG > 0 ? st[7] - Bt[0] : -st[7] - Bt[0];
@@ -757,7 +758,7 @@ __device__ __forceinline__ void flux64_item(const Dims& g, int d, const double* 
             gh[11] = B[0] + SG * col[(11 * SL + slot) * NT];
         }
         if (vbar && vbar[0]) {
-            const double iW = rcp_pos(W);
+            const double iW = rcp_wide(W);
             vh[0] = pr[2] * iW;
             vh[1] = pr[3] * iW;
         }
@@ -1355,7 +1356,7 @@ __device__ __forceinline__ void cell_sources(const Dims& g, const double* const*
     for (int i = 0; i < 3; i++) u[i] = prim[1 + i][o];
     const double u2 = fma(u[0], u[0], fma(u[1], u[1], u[2] * u[2]));
     const double xw = M ? fma(p4, u2, 1.0) : 1.0 + u2;
-    const double iW = rsqrt_ge1(xw);
+    const double iW = rsqrt_wide(xw);
     // Gauss law: sqrt(gamma) rho_e = div q_E by central differences
     double divqE = 0.0;
 #pragma unroll

@@ -1,7 +1,9 @@
 """The per-cell device code (csrc/*.cuh) compiled as plain C++ (device_on_host.h) and run on
 the CPU at inputs where a rule inside it can go wrong."""
+import math
 import shutil
 import subprocess
+from decimal import Decimal, getcontext
 from fractions import Fraction as Fr
 from pathlib import Path
 
@@ -154,3 +156,48 @@ def test_momentum_source_of_a_cold_gas(run):
         u2, U = psi ** 4 * 6 * f * f, (psi ** 4 * 6 * f * f + 6 * f * f / psi ** 8) / 2
         want = psi ** 6 * 2 * (Fr(1, 4) * 2 / psi) * ((rho + 4 * p) * u2 + 3 * p + U)
         assert abs(Fr(got) - want) <= want / 10 ** 14
+
+
+# the Lorentz factor of an HLL half; the transport velocity u^t / W of a uniform state at a face;
+# the charge-current source -div q_E u^t / W
+LORENTZ = GRID + r"""
+int main() {
+    double u;
+    while (std::scanf("%la", &u) == 1) {
+        const Dims g = grid4();
+        const double st[8] = {1, u, 2 * u, 2 * u, 1, 0.1, 0.2, 0.3}, Bt[2] = {0.5, 0.25};
+        double gh[8], W, A[11][8], F[8][8], vb[2][8], src[8];
+        const double *prim[8], *bf[3];
+        double *Fp[8], *vbar[2] = {vb[0], vb[1]};
+        hll_half64<1>(st, Bt, 0.5, 0.125, 4.0, gh, W);
+        for (int c = 0; c < 8; c++)
+            for (int v = 0; v < 11; v++) A[v][c] = v < 8 ? st[v] : 0.5;
+        for (int v = 0; v < 8; v++) {
+            prim[v] = A[v];
+            Fp[v] = F[v];
+        }
+        for (int d = 0; d < 3; d++) bf[d] = A[8 + d];
+        static double sm[Flux64<false, false>::SM];
+        flux64_item<false, false, false>(g, 0, prim, bf, nullptr, nullptr, nullptr, Fp, vbar, nullptr, sm, 1);
+        for (int c = 0; c < 8; c++) A[5][c] = c;   // d_x E^x = 4
+        const int c[3] = {4, 0, 0};
+        cell_sources<false, false>(g, prim, bf, nullptr, nullptr, nullptr, c, 4, src);
+        std::printf("%a %a %a\n", W, vb[0][3], src[6]);
+    }
+}
+"""
+
+
+def test_lorentz_factor_at_any_velocity(run):
+    """W = sqrt(1 + u^2) and u^t / W over the whole range of FP64 squares, also where 1 + u^2 or W
+    leaves the range of the FP32 estimates (u = 6e18 and 3e37): two ulp each."""
+    us = [0.0, 1e-3, 1.0, 1e9, 4e18, 8e18, 1e25, 2e37, 5e37, 1e100, 1e150]
+    getcontext().prec = 40
+    for u, (W, v, s) in zip(us, run(LORENTZ, [[u] for u in us])):
+        want = (1 + 9 * Decimal(u) ** 2).sqrt()
+        tol = Decimal(2) ** -51
+        assert abs(Decimal(W) - want) <= tol * want
+        assert abs(Decimal(v) - 2 * Decimal(u) / want) <= tol
+        assert abs(Decimal(s) + 8 * Decimal(u) / want) <= 4 * tol
+    bad = run(LORENTZ, [[float("nan")], [1e200]])
+    assert all(math.isnan(r[0]) for r in bad)   # (the square of 1e200 is infinite)
