@@ -218,11 +218,14 @@ __device__ __forceinline__ double mg_block_sum(double v, double* sh)
     return sh[32];
 }
 
-// the block sum where one warp holds every value: five shuffles, no barrier
+// the block sum where one warp holds every value: five shuffles.  Shuffles order no memory, so a
+// warp barrier stands before them: what the lanes wrote before the sum is read after it by
+// others (the search direction), as with the barriers of the block sum.
 template <bool W>
 __device__ __forceinline__ double mg_sum(double v, double* sh)
 {
     if (!W) return mg_block_sum(v, sh);
+    __syncwarp();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;

@@ -44,4 +44,4 @@ inline double rsqrt(double a) { return 1.0 / std::sqrt(a); }
 inline unsigned __umulhi(unsigned a, unsigned b) { return (unsigned)((uint64_t)a * b >> 32); }
 template <class T> inline T atomicAdd(T* p, T v) { T o = *p; *p += v; return o; }
 struct Idx3 { unsigned x, y, z; };
-inline Idx3 threadIdx{0, 0, 0}, blockIdx{0, 0, 0}, blockDim{1, 1, 1}, gridDim{1, 1, 1};
+inline thread_local Idx3 threadIdx{0, 0, 0}, blockIdx{0, 0, 0}, blockDim{1, 1, 1}, gridDim{1, 1, 1};
