@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(1024) k_mg_tail(MgTail T, MgArgs m, double* __
 {
     grid_dep_sync();
     extern __shared__ double tail_sm[];
-    __shared__ double sh[33];
+    __shared__ double sh[kMgSums];
     if (T.smem) {
         const MgLevel G = T.lev[T.first];
         const MgLevel L = tail_level(T, T.first, tail_sm);
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(256) k_mg_up2(MgLevel L, MgLevel C, MgArgs m)
 __global__ void __launch_bounds__(256) k_mg_div(Dims g, CP3 bq, int cc, MgLevel L, MgArgs m, double* __restrict__ part)
 {
     grid_dep_sync();
-    __shared__ double sh[33];
+    __shared__ double sh[kMgSums];
     double s = 0.0;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < L.cells;
          t += (long long)gridDim.x * blockDim.x) {
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(256) k_mg_mean(const double* __restrict__ part
                                                  long long cells)
 {
     grid_dep_sync();
-    __shared__ double sh[33];
+    __shared__ double sh[kMgSums];
     double s = 0.0;
     for (int b = threadIdx.x; b < nb; b += blockDim.x) s += part[b];
     s = mg_block_sum(s, sh);

@@ -12,8 +12,10 @@ constexpr long long kMgMaxCoarse = 4096;   // cells of the coarsest level (one t
 constexpr long long kMgBlockCells = 1024;  // levels this small run inside one thread block
                                            // (one SM does 2 FP64 FMA per cycle: larger
                                            // levels are faster as grid-wide launches)
-constexpr size_t kMgTailSmem = 48 * 1024;  // the block keeps its levels in shared memory
-                                           // when they fit in this many bytes
+constexpr int kMgSums = 33;                // shared doubles of a block sum
+constexpr size_t kMgTailSmem = 48 * 1024 - 8 * (kMgSums + 1);  // the block keeps its levels in
+                                           // shared memory when they fit in this many bytes: a
+                                           // block's 48 KB less those of its sums
 constexpr int kMgParts = 1024;             // partial sums of the mean
 
 // one cell-centred level (no ghosts, x fastest)

@@ -299,3 +299,69 @@ def test_one_warp_coarse_solve(run, n0, n1, bc):
     e = np.pad(phi, 1, mode=mode)
     lap = 4.0 * (e[1:-1, 2:] - 2 * phi + e[1:-1, :-2]) + (e[2:, 1:-1] - 2 * phi + e[:-2, 1:-1])
     assert np.abs(lap - (rhs - rhs.mean())).max() <= 1e-12
+
+
+# mg_clean with the CUDA runtime's launch call replaced: each launch's grid, block and shared bytes
+# are printed, and launch `bad` (counted from 0; -1: none) is refused
+LAUNCHES = r"""
+#include <cstdio>
+#include <cuda_runtime.h>
+static int launched, bad;
+static const void* fn[4096];
+extern "C" cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* k, void**)
+{
+    if (launched == bad) return launched++, cudaErrorInvalidValue;
+    fn[launched++] = k;
+    for (size_t v : {(size_t)c->gridDim.x, (size_t)c->gridDim.y, (size_t)c->gridDim.z, (size_t)c->blockDim.x,
+                     c->dynamicSmemBytes})
+        std::printf("%a ", (double)v);
+    return cudaSuccess;
+}
+inline void __syncthreads() {}
+inline void __syncwarp() {}
+inline double __shfl_xor_sync(unsigned, double v, int) { return v; }
+inline double __shfl_down_sync(unsigned, double v, int) { return v; }
+extern "C" cudaError_t cudaGetLastError() { return cudaSuccess; }
+#undef __shared__
+#define __shared__
+#define asm
+#define volatile(...)   // (griddepcontrol)
+#include "elliptic.cu"
+namespace grmhd { thread_local bool launch_overlap; namespace { double tail_sm[1]; } }
+using namespace grmhd;
+int main() {
+    double n[3], b;
+    while (std::scanf("%la %la %la %la", n, n + 1, n + 2, &b) == 4) {
+        Dims g = {};
+        for (int d = 0; d < 3; d++) {
+            g.n[d] = (int)n[d];
+            g.act[d] = n[d] > 1;
+            g.idx[d] = g.act[d];
+        }
+        set_divisors(g);
+        launched = 0;
+        bad = (int)b;
+        MgPlan plan;
+        double *bq[3] = {}, scratch[1];
+        if (mg_plan(g, &plan) != 0) return 1;
+        long long nl = 0;
+        const cudaError_t e = mg_clean(g, plan, scratch, scratch, scratch, bq, false, 2, 152, nullptr, &nl);
+        std::printf("%a %a %a\n", (double)e, (double)launched, (double)(fn[launched - 1] == (const void*)k_mg_correct));
+    }
+}
+"""
+
+
+def launches(run, n, bad=-1):
+    r = [int(x) for x in run(LAUNCHES, [[*n, *[1] * (3 - len(n)), bad]])[0]]
+    return [r[i:i + 5] for i in range(0, len(r) - 3, 5)], r[-3:]
+
+
+@pytest.mark.parametrize("n", [(35, 35), (34, 36), (70, 70), (560, 560), (1120, 1120), (36, 34), (1223,), (9784,),
+                               (17, 9, 8), (512, 512), (48, 48, 48)])
+def test_cleaning_launches_fit_a_block(run, n):
+    """Every launch's shared memory fits the 48 KB that a block has without opting in: the tail
+    kernel's dynamic bytes with its static block sums (33 doubles, to the next 16 bytes)."""
+    ls, (err, _, last) = launches(run, n)
+    assert err == 0 and last == 1
+    assert all(dyn + (33 * 8 + 8 if block == 1024 else 0) <= 48 * 1024 for *_, block, dyn in ls)
