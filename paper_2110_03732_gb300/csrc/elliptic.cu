@@ -706,7 +706,15 @@ size_t mg_scratch_bytes(const MgPlan& p)
 cudaError_t mg_clean(const Dims& g, const MgPlan& plan0, double* scratch, double* alt0, double* alt1,
                      double* const* bq, bool cc, int cycles, int nsm, cudaStream_t st, long long* launches)
 {
+    // launches, up to the first that is refused: what comes after one, the field's correction
+    // above all, would work on a level that was not computed
     long long nl = 0;
+    cudaError_t err = cudaSuccess;
+    auto go = [&](auto* k, dim3 grid, int block, size_t smem, auto&&... args) {
+        if (err != cudaSuccess) return;
+        nl++;
+        err = launch_dyn(k, grid, block, smem, st, args...);
+    };
     MgPlan plan = plan0;
     const long long T = plan.total;
     const long long nc = plan.lev[plan.nlev - 1].cells;
@@ -734,12 +742,9 @@ cudaError_t mg_clean(const Dims& g, const MgPlan& plan0, double* scratch, double
         pq.p[d] = bq[d];
     }
     const int nb = (int)((F.cells + 255) / 256 < kMgParts ? (F.cells + 255) / 256 : kMgParts);
-    nl++;
-    launch_k(k_mg_div, nb, 256, st, g, cq, cc ? 1 : 0, F, m, part);
-    nl++;
-    launch_k(k_mg_mean, 1, 256, st, (const double*)part, nb, mean, F.cells);
-    nl++;
-    launch_k(k_mg_sub_mean, mg_grid(F.cells, nsm), 256, st, F, (const double*)mean);
+    go(k_mg_div, nb, 256, 0, g, cq, cc ? 1 : 0, F, m, part);
+    go(k_mg_mean, 1, 256, 0, (const double*)part, nb, mean, F.cells);
+    go(k_mg_sub_mean, mg_grid(F.cells, nsm), 256, 0, F, (const double*)mean);
     const int cg_it = (int)(2 * nc + 20);
     // levels of at most kMgBlockCells cells run inside one block (k_mg_tail)
     MgTail tail;
@@ -763,52 +768,43 @@ cudaError_t mg_clean(const Dims& g, const MgPlan& plan0, double* scratch, double
         for (int l = 0; l < tail.first; l++) {
             const MgLevel& L = plan.lev[l];
             if (tiled) {
-                nl++;
                 const int T = tile_side(L);
                 const dim3 gr((L.n[0] + T - 1) / T, (L.n[1] + T - 1) / T);
-                launch_dyn(T == 32 ? k_mg_down2<32> : k_mg_down2<16>, gr, 256, 0, st, L, plan.lev[l + 1], m,
+                go(T == 32 ? k_mg_down2<32> : k_mg_down2<16>, gr, 256, 0, L, plan.lev[l + 1], m,
                            (cyc == 0 || l > 0) ? 1 : 0);
                 continue;
             }
             const int bs = mg_grid(half_items(L), nsm);
             for (int s = 0; s < 2; s++) {
-                nl++;
-                launch_k(k_mg_smooth, bs, 256, st, L, m, 0);
-                nl++;
-                launch_k(k_mg_smooth, bs, 256, st, L, m, 1);
+                go(k_mg_smooth, bs, 256, 0, L, m, 0);
+                go(k_mg_smooth, bs, 256, 0, L, m, 1);
             }
-            nl++;
-            launch_k(k_mg_restrict, mg_grid(plan.lev[l + 1].cells, nsm), 256, st, L, plan.lev[l + 1], m);
+            go(k_mg_restrict, mg_grid(plan.lev[l + 1].cells, nsm), 256, 0, L, plan.lev[l + 1], m);
         }
         // the small levels and the coarsest solve (from zero); with a single level this
         // is the whole solve, and further cycles would repeat it
-        nl++;
-        launch_dyn(k_mg_tail, dim3(1), 1024, tail_dyn, st, tail, m, cg_r, cg_p, cg_q, cg_it);
+        go(k_mg_tail, 1, 1024, tail_dyn, tail, m, cg_r, cg_p, cg_q, cg_it);
         if (plan.nlev == 1) break;
         for (int l = tail.first - 1; l >= 0; l--) {
             const MgLevel& L = plan.lev[l];
             if (tiled) {
-                nl++;
                 const int T = tile_side(L);
                 const dim3 gr((L.n[0] + T - 1) / T, (L.n[1] + T - 1) / T);
-                launch_dyn(T == 32 ? k_mg_up2<32> : k_mg_up2<16>, gr, 256, 0, st, L, plan.lev[l + 1], m);
+                go(T == 32 ? k_mg_up2<32> : k_mg_up2<16>, gr, 256, 0, L, plan.lev[l + 1], m);
                 continue;
             }
             const int b = mg_grid(L.cells, nsm), bs = mg_grid(half_items(L), nsm);
-            nl++;
-            launch_k(k_mg_prolong, b, 256, st, L, plan.lev[l + 1], m);
+            go(k_mg_prolong, b, 256, 0, L, plan.lev[l + 1], m);
             for (int s = 0; s < 2; s++) {
-                nl++;
-                launch_k(k_mg_smooth, bs, 256, st, L, m, 0);
-                nl++;
-                launch_k(k_mg_smooth, bs, 256, st, L, m, 1);
+                go(k_mg_smooth, bs, 256, 0, L, m, 0);
+                go(k_mg_smooth, bs, 256, 0, L, m, 1);
             }
         }
     }
-    nl++;
-    launch_k(k_mg_correct, mg_grid(F.cells, nsm), 256, st, g, pq, cc ? 1 : 0, F, m);
+    go(k_mg_correct, mg_grid(F.cells, nsm), 256, 0, g, pq, cc ? 1 : 0, F, m);
     if (launches) *launches += nl;
-    return cudaGetLastError();
+    const cudaError_t last = cudaGetLastError();   // (read in any case: it clears the error)
+    return err != cudaSuccess ? err : last;
 }
 
 GRMHD_OOB_READER(oob_elliptic)

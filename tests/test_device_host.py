@@ -365,3 +365,12 @@ def test_cleaning_launches_fit_a_block(run, n):
     ls, (err, _, last) = launches(run, n)
     assert err == 0 and last == 1
     assert all(dyn + (33 * 8 + 8 if block == 1024 else 0) <= 48 * 1024 for *_, block, dyn in ls)
+
+
+def test_cleaning_stops_at_a_refused_launch(run):
+    """A refused launch ends the cleaning with its error: the field is not corrected by a
+    potential that was not solved for."""
+    total = len(launches(run, (96, 64))[0])
+    for bad in range(total):
+        _, (err, launched, last) = launches(run, (96, 64), bad)
+        assert err == 1 and launched == bad + 1 and last == 0
