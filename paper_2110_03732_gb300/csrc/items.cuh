@@ -295,8 +295,8 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
         evaluate_accept(Dn, mul(a.qb.p[4][id], ip6), S, Es, B, etat, g.igh, emode, u, e);
         const double fm = from_hi(max(mag_hi(e.f[0]), max(mag_hi(e.f[1]), mag_hi(e.f[2]))));
         // (every comparison is false for a NaN; a momentum scale that has left the range of FP32
-        // accepts nothing)
-        if (!ok || !(rt.M > 0.0f) || !(rt.M < 1e30f) || !(fm <= a.tol * f2d_int(rt.M)) || !pos_int(e.wt) || !mag_below_int(e.W, kHi1e10)) {
+        // accepts nothing, and a scale of zero, a cell at rest, accepts a residual of zero)
+        if (!ok || !(rt.M < 1e30f) || !(fm <= a.tol * f2d_int(rt.M)) || !pos_int(e.wt) || !mag_below_int(e.W, kHi1e10)) {
             implicit_general<M, CC, ACC>(g, a, t);
             return;
         }

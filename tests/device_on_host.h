@@ -6,7 +6,7 @@
 #define __host__
 #define __global__
 #define __forceinline__ inline
-#define __noinline__
+#define __noinline__ __attribute__((noinline))
 #define __launch_bounds__(...)
 #define __grid_constant__
 #include <algorithm>

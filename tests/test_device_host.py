@@ -22,13 +22,13 @@ def run(tmp_path_factory):
     """The rows (lists of floats) through the program `src`, a list of floats back for each."""
     built = {}
 
-    def call(src, rows):
+    def call(src, rows, *flags):
         if src not in built:
             d = tmp_path_factory.mktemp("device")
             (d / "t.cpp").write_text('#include "device_on_host.h"\n' + src)
             inc = [ROOT / "tests", CUDA, ROOT / "paper_2110_03732_gb300" / "csrc", ROOT / "include"]
             subprocess.run(["g++", "-O1", "-std=c++17", "-ffp-contract=off", "-pthread", "-ffunction-sections",
-                            "-Wl,--gc-sections", *(f"-I{i}" for i in inc), str(d / "t.cpp"),
+                            "-Wl,--gc-sections", *flags, *(f"-I{i}" for i in inc), str(d / "t.cpp"),
                             "-o", str(d / "t")], check=True)
             built[src] = d / "t"
         text = "\n".join(" ".join(float(x).hex() for x in r) for r in rows) + "\n"
@@ -59,13 +59,23 @@ Dims grid4()
 }
 """
 
-# the conserved variables of a state in a flat cell, and the solve from another start
+# a state in a flat cell and its solve from another start: prints the failures, rho, u and p, and
+# how often the general solve and the double-word corrections were entered (with
+# -finstrument-functions)
 IMPLICIT = GRID + r"""
+static int general, refine;
+#define HOOK extern "C" __attribute__((no_instrument_function)) void
+HOOK __cyg_profile_func_exit(void*, void*) {}
+HOOK __cyg_profile_func_enter(void* f, void*)
+{
+    general += f == (void*)implicit_general<false, false, ACC>;
+    refine += f == (void*)newton_refine_dw<ACC>;
+}
 int main() {
-    double s, r, a_dt;   // density scale, field scale (r r = s), a_ii dt
-    while (std::scanf("%la %la %la", &s, &r, &a_dt) == 3) {
+    double s, r, a_dt, us, u0;   // density scale, field scale, a_ii dt, velocity scale, start
+    while (std::scanf("%la %la %la %la %la", &s, &r, &a_dt, &us, &u0) == 5) {
         const Dims g = grid4();
-        const double rho = 1.3 * s, p = 0.7 * s, u[3] = {0.4, -0.6, 0.3}, E[3] = {0.5 * r, 0.2 * r, -0.3 * r},
+        const double rho = 1.3 * s, p = 0.7 * s, u[3] = {0.4 * us, -0.6 * us, 0.3 * us}, E[3] = {0.5 * r, 0.2 * r, -0.3 * r},
                      B[3] = {0.6 * r, -0.8 * r, 0.5 * r};
         const double W = std::sqrt(1 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]), hW = (rho + 4.0 * p) * W;
         double q[8], U = 0;
@@ -84,7 +94,7 @@ int main() {
             a.qb.p[v] = A[v];
             a.prim.p[v] = A[11 + v];
         }
-        const double start[8] = {s, 0.1, 0.1, 0.1, s, 0, 0, 0};
+        const double start[8] = {s, u0, u0, u0, s, 0, 0, 0};
         for (int c = 0; c < 8; c++)
             for (int v = 0; v < 8; v++) A[11 + v][c] = start[v];
         for (int d = 0; d < 3; d++) {
@@ -99,15 +109,27 @@ int main() {
         a.ia_dt = a_dt > 0 ? 1 / a_dt : 0;
         a.stiff = a_dt > 0;
         a.ighf = 0.25f;
-        a.kmax = 50;
+        a.kmax = 100;
         a.tol = 1e-13;
         a.tolf = 1e-13f;
         a.nfail = &nfail;
-        implicit_item<false, false, false>(g, a, 1);
-        std::printf("%a %a %a %a %a %a\n", (double)nfail, A[11][3] / s, A[12][3], A[13][3], A[14][3], A[15][3] / s);
+        if (ACC) {
+            static float f32[11][8];
+            for (int v = 0; v < 11; v++) a.p32.p[v] = f32[v];
+            a.tol = 1e-10;
+            a.tolf = 1e-10f;
+        }
+        general = refine = 0;
+        implicit_item<false, false, ACC>(g, a, 1);
+        std::printf("%a %a %a %a %a %a %a %a\n", (double)nfail, A[11][3] / s, A[12][3], A[13][3], A[14][3], A[15][3] / s,
+                    (double)general, (double)refine);
     }
 }
 """
+
+
+def implicit(run, rows, acc=False):
+    return run(IMPLICIT.replace("ACC", str(acc).lower()), rows, "-finstrument-functions")
 
 
 @pytest.mark.parametrize("a_dt", [0.0, 0.05])
@@ -117,12 +139,21 @@ def test_implicit_solve_at_any_scale(run, a_dt):
     the momentum leaves the range of FP32.  1e-11: the 1e-13 of the residual test on both
     sides, and the condition of this state (below 10)."""
     r = [2.0 ** k for k in (0, -40, 40, 64, 70, 100)]
-    rows = run(IMPLICIT, [[x * x, x, a_dt] for x in r])
+    rows = implicit(run, [[x * x, x, a_dt, 1.0, 0.1] for x in r])
     assert all(row[0] == 0 for row in rows)
     if a_dt == 0.0:   # E held fixed: the state itself is the root
-        assert rows[0][1:] == pytest.approx([1.3, 0.4, -0.6, 0.3, 0.7], rel=1e-11)
+        assert rows[0][1:6] == pytest.approx([1.3, 0.4, -0.6, 0.3, 0.7], rel=1e-11)
     for row in rows[1:]:
-        assert row[1:] == pytest.approx(rows[0][1:], rel=1e-11)
+        assert row[1:6] == pytest.approx(rows[0][1:6], rel=1e-11)
+
+
+@pytest.mark.parametrize("a_dt", [0.0, 0.05])
+def test_cell_at_rest_takes_the_direct_path(run, a_dt):
+    """A cell without momentum has the momentum scale zero: its start u = 0 solves it exactly, and
+    the direct path accepts that."""
+    for row in implicit(run, [[s, 0.0, a_dt, 0.0, 0.0] for s in (1.0, 1e-12, 1e6)]):
+        assert row[:1] + row[2:5] == [0.0] * 4 and row[1::4] == pytest.approx([1.3, 0.7], rel=1e-14)
+        assert row[6] == 0
 
 
 # the sources of a cell on a metric with psi alone
