@@ -1471,11 +1471,12 @@ __device__ __forceinline__ bool newton_refine_dw(const CellDW& c, dw* u, float t
 // bounded step).  u: in = initial guess, out = solution.  Converged when |f| is at
 // `tol` against its own momentum scale M, or when the step no longer moves u.
 // Returns iterations, or -1.  uin: the FP32 value of the start when the caller has it
-// (has_uin; the start is then exactly that value).  ACC: double-word acceptance (the
-// mixed-precision path, whose tolerance is at least 1e-11; see newton_refine_dw).
+// (has_uin; the start is then exactly that value).  refined: u is where the double-word
+// corrections have ended already.  ACC: double-word acceptance (the mixed-precision path,
+// whose tolerance is at least 1e-11; see newton_refine_dw).
 template <bool ACC = false>
 __device__ __forceinline__ int newton_solve(const CellIn& c, double* u, Eval& e, int kmax, double tol, float tolf,
-                                            bool has_uin, const F3& uin)
+                                            bool has_uin, const F3& uin, bool refined = false)
 {
     const CellF cf = cell_f32(c);
     // the FP32 first step saves an FP64 evaluation only when the tolerance lies below
@@ -1483,7 +1484,9 @@ __device__ __forceinline__ int newton_solve(const CellIn& c, double* u, Eval& e,
     // 1e-13, not the mixed path's 1e-10
     F3 uf1 = uin;   // FP32 value of u at the first direction (when has1)
     bool has1 = has_uin;
-    if (c.emode != 2) {
+    if (refined) {
+        has1 = false;
+    } else if (c.emode != 2) {
         // Newton corrections from the double-word residual; the FP64 residual below
         // then accepts the root (or, with ACC, the double-word one already did), or the
         // FP64 iteration continues from there

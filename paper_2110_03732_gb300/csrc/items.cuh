@@ -60,11 +60,14 @@ __device__ __forceinline__ void implicit_f32(double rho, double pres, const doub
 // The general solve of one cell (cells that implicit_item's direct path does not accept,
 // and the dynamo form): a call, so that its FP64 iteration takes neither registers nor
 // instruction-cache room from the direct path.
+// refined: the direct path's double-word corrections have ended at (r0, r1, r2), and the
+// solve goes on from there (from its start where that is not finite) without repeating them.
 // CC: the magnetic field is cell-centred (a.bf holds cell q_B, GLM variant) instead of
 // staggered on faces.  ACC: the mixed-precision path, whose double-word residual
 // accepts the root (newton_refine_dw)
 template <bool M, bool CC, bool ACC>
-__device__ __noinline__ void implicit_general(const Dims& g, const ImpArgs& a, long long t)
+__device__ __noinline__ void implicit_general(const Dims& g, const ImpArgs& a, long long t, bool refined = false,
+                                              double r0 = 0.0, double r1 = 0.0, double r2 = 0.0)
 {
     // flat metric: alpha = psi = 1 known at compile time
     const double* __restrict__ psi = M ? a.psi : nullptr;
@@ -128,7 +131,12 @@ __device__ __noinline__ void implicit_general(const Dims& g, const ImpArgs& a, l
             if (!mag_below_int(u[i], kHi1e30)) fin = false;   // also NaN
         }
         if (!fin) u[0] = u[1] = u[2] = 0.0;
-        int it = newton_solve<ACC>(ci, u, e, kmax, tol, a.tolf, hist && fin, ust);
+        if (refined && finite_int(r0) && finite_int(r1) && finite_int(r2)) {
+            u[0] = r0;
+            u[1] = r1;
+            u[2] = r2;
+        }
+        int it = newton_solve<ACC>(ci, u, e, kmax, tol, a.tolf, hist && fin, ust, refined);
         if (it < 0 && fin) {
             u[0] = u[1] = u[2] = 0.0;
             it = newton_solve<ACC>(ci, u, e, kmax, tol, a.tolf, false, ust);
@@ -263,7 +271,7 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
     float f32[11], uh[3];
     if (ACC) {
         if (!acc) {
-            implicit_general<M, CC, ACC>(g, a, t);
+            implicit_general<M, CC, ACC>(g, a, t, ok, dw_to_double(ud[0]), dw_to_double(ud[1]), dw_to_double(ud[2]));
             return;
         }
         const double iW = dw_finite(dw_rcp(rt.W));
@@ -297,7 +305,7 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
         // (every comparison is false for a NaN; a momentum scale that has left the range of FP32
         // accepts nothing, and a scale of zero, a cell at rest, accepts a residual of zero)
         if (!ok || !(rt.M < 1e30f) || !(fm <= a.tol * f2d_int(rt.M)) || !pos_int(e.wt) || !mag_below_int(e.W, kHi1e10)) {
-            implicit_general<M, CC, ACC>(g, a, t);
+            implicit_general<M, CC, ACC>(g, a, t, ok, u[0], u[1], u[2]);
             return;
         }
         const double rho = Dn * e.iW, pres = fma(e.wt, e.iW, -rho) * g.igh;

@@ -156,6 +156,20 @@ def test_cell_at_rest_takes_the_direct_path(run, a_dt):
         assert row[6] == 0
 
 
+@pytest.mark.parametrize("acc", [False, True])
+@pytest.mark.parametrize("a_dt", [0.0, 0.05])
+def test_refused_cell_goes_on_from_the_corrections(run, a_dt, acc):
+    """A cell whose double-word corrections do not reach the root goes on in FP64 from where they
+    ended: they run once.  (The result: to the residual's tolerance times the condition of w_t in
+    the velocity at u = 20, W^2 = 400.)"""
+    rows = implicit(run, [[1.0, 1.0, a_dt, 20.0, x] for x in (0.0, 0.01)], acc)
+    near = implicit(run, [[1.0, 1.0, a_dt, 20.0, rows[0][2]]], acc)[0]
+    for row in rows:
+        assert row[0] == 0 and row[1:6] == pytest.approx(near[1:6], rel=4e-8 if acc else 4e-11)
+    assert any(row[6] == 1 for row in rows)
+    assert all(row[7] == 1 for row in rows)
+
+
 # the sources of a cell on a metric with psi alone
 SOURCES = GRID + r"""
 int main() {
