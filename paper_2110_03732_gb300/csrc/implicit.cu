@@ -36,12 +36,39 @@ __global__ void __launch_bounds__(128, 8) k_implicit_cc(const __grid_constant__ 
         implicit_item<M, true>(g, a, t);
 }
 
+// The dynamo form (xi != 0): every cell takes the general solve, inline and with the registers
+// that its FP64 iteration wants (96, five blocks per SM).  As a call from k_implicit's 72
+// registers it was slower: 384^2 FP64 152 against 184 us, mixed 158 / 182, 64^3 with a metric
+// 287 / 305, 1-D of 4096 cells 45 / 52.
+template <bool M, bool CC, bool ACC>
+__global__ void __launch_bounds__(128, CC ? 4 : 5) k_implicit_dynamo(const __grid_constant__ Dims g,
+                                                                    const __grid_constant__ ImpArgs a)
+{
+    grid_dep_sync();
+    const long long tot = (long long)g.n[0] * g.n[1] * g.n[2];
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot;
+         t += (long long)gridDim.x * blockDim.x)
+        implicit_solve<M, CC, ACC>(g, a, t, false, 0.0, 0.0, 0.0);
+}
+
+template <bool M, bool ACC>
+static auto implicit_kernel(const ImpArgs& a)
+{
+    return a.xi != 0.0 ? k_implicit_dynamo<M, false, ACC> : k_implicit<M, ACC>;
+}
+
+template <bool M>
+static auto implicit_kernel_cc(const ImpArgs& a)
+{
+    return a.xi != 0.0 ? k_implicit_dynamo<M, true, false> : k_implicit_cc<M>;
+}
+
 cudaError_t launch_implicit(const Dims& g, const ImpArgs& a, int nsm, cudaStream_t st)
 {
     const long long work = (long long)g.n[0] * g.n[1] * g.n[2];
     const bool m = a.psi || a.alp;
-    if (a.dwacc) launch_k(m ? k_implicit<true, true> : k_implicit<false, true>, grid_for(work, 128, nsm), 128, st, g, a);
-    else launch_k(m ? k_implicit<true, false> : k_implicit<false, false>, grid_for(work, 128, nsm), 128, st, g, a);
+    if (a.dwacc) launch_k(m ? implicit_kernel<true, true>(a) : implicit_kernel<false, true>(a), grid_for(work, 128, nsm), 128, st, g, a);
+    else launch_k(m ? implicit_kernel<true, false>(a) : implicit_kernel<false, false>(a), grid_for(work, 128, nsm), 128, st, g, a);
     return cudaGetLastError();
 }
 
@@ -49,8 +76,8 @@ cudaError_t launch_implicit_cc(const Dims& g, const ImpArgs& a, int nsm, cudaStr
 {
     const long long work = (long long)g.n[0] * g.n[1] * g.n[2];
     // GLM contexts are FP64 only: the FP64 residual accepts the root
-    launch_k(a.psi || a.alp ? k_implicit_cc<true> : k_implicit_cc<false>, grid_for(work, 128, nsm), 128, st, g,
-             a);
+    launch_k(a.psi || a.alp ? implicit_kernel_cc<true>(a) : implicit_kernel_cc<false>(a), grid_for(work, 128, nsm), 128,
+             st, g, a);
     return cudaGetLastError();
 }
 

@@ -58,16 +58,15 @@ __device__ __forceinline__ void implicit_f32(double rho, double pres, const doub
 }
 
 // The general solve of one cell (cells that implicit_item's direct path does not accept,
-// and the dynamo form): a call, so that its FP64 iteration takes neither registers nor
-// instruction-cache room from the direct path.
+// and the dynamo form).
 // refined: the direct path's double-word corrections have ended at (r0, r1, r2), and the
 // solve goes on from there (from its start where that is not finite) without repeating them.
 // CC: the magnetic field is cell-centred (a.bf holds cell q_B, GLM variant) instead of
 // staggered on faces.  ACC: the mixed-precision path, whose double-word residual
 // accepts the root (newton_refine_dw)
 template <bool M, bool CC, bool ACC>
-__device__ __noinline__ void implicit_general(const Dims& g, const ImpArgs& a, long long t, bool refined = false,
-                                              double r0 = 0.0, double r1 = 0.0, double r2 = 0.0)
+__device__ __forceinline__ void implicit_solve(const Dims& g, const ImpArgs& a, long long t, bool refined, double r0,
+                                               double r1, double r2)
 {
     // flat metric: alpha = psi = 1 known at compile time
     const double* __restrict__ psi = M ? a.psi : nullptr;
@@ -180,6 +179,18 @@ __device__ __noinline__ void implicit_general(const Dims& g, const ImpArgs& a, l
     implicit_store<M>(a, id, rho, pres, u, e.E, ip2, p4, qEs, f32, atmo ? nullptr : uh);
 }
 
+// the same as a call, so that its FP64 iteration takes neither registers nor
+// instruction-cache room from the direct path
+template <bool M, bool CC, bool ACC>
+__device__ __noinline__ void implicit_general(const Dims& g, const ImpArgs& a, long long t, bool refined = false,
+                                              double r0 = 0.0, double r1 = 0.0, double r2 = 0.0)
+{
+    implicit_solve<M, CC, ACC>(g, a, t, refined, r0, r1, r2);
+}
+
+// the dynamo form (xi != 0), which has no direct path
+__device__ __forceinline__ bool has_dynamo(const ImpArgs& a) { return (__double_as_longlong(a.xi) << 1) != 0; }
+
 // One cell: the direct path takes the double-word Newton corrections from the kept start
 // and accepts their root by the FP64 residual (ACC: the double-word one); atmosphere cells
 // are written at once; everything else is implicit_general's.  The FP64 inputs are split
@@ -191,7 +202,7 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
     int c[3];
     interior_coords(g, t, c);
     const long long id = lin(g, c[0], c[1], c[2]);
-    if ((__double_as_longlong(a.xi) << 1) != 0) {   // the dynamo form (xi != 0)
+    if (has_dynamo(a)) {
         implicit_general<M, CC, ACC>(g, a, t);
         return;
     }

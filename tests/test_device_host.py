@@ -27,7 +27,7 @@ def run(tmp_path_factory):
             d = tmp_path_factory.mktemp("device")
             (d / "t.cpp").write_text('#include "device_on_host.h"\n' + src)
             inc = [ROOT / "tests", CUDA, ROOT / "paper_2110_03732_gb300" / "csrc", ROOT / "include"]
-            subprocess.run(["g++", "-O1", "-std=c++17", "-ffp-contract=off", "-pthread", "-ffunction-sections",
+            subprocess.run(["g++", "-O0", "-std=c++17", "-ffp-contract=off", "-pthread", "-ffunction-sections",
                             "-Wl,--gc-sections", *flags, *(f"-I{i}" for i in inc), str(d / "t.cpp"),
                             "-o", str(d / "t")], check=True)
             built[src] = d / "t"
@@ -168,6 +168,49 @@ def test_refused_cell_goes_on_from_the_corrections(run, a_dt, acc):
         assert row[0] == 0 and row[1:6] == pytest.approx(near[1:6], rel=4e-8 if acc else 4e-11)
     assert any(row[6] == 1 for row in rows)
     assert all(row[7] == 1 for row in rows)
+
+
+# which kernel the implicit solve launches for (psi set, xi, mixed precision, cell-centred field)
+KERNELS = r"""
+#include <cuda_runtime.h>
+static const void* fn;
+extern "C" cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void* k, void**)
+{
+    fn = k;
+    return cudaSuccess;
+}
+extern "C" cudaError_t cudaGetLastError() { return cudaSuccess; }
+#define asm
+#define volatile(...)   // (griddepcontrol)
+""" + GRID + r"""
+#include "implicit.cu"
+namespace grmhd { thread_local bool launch_overlap; }
+int main() {
+    double m, xi, acc, cc;
+    while (std::scanf("%la %la %la %la", &m, &xi, &acc, &cc) == 4) {
+        const Dims g = grid4();
+        ImpArgs a = {};
+        double psi;
+        a.psi = m ? &psi : nullptr;
+        a.xi = xi;
+        a.dwacc = (int)acc;
+        if (cc) launch_implicit_cc(g, a, 152, nullptr);
+        else launch_implicit(g, a, 152, nullptr);
+        const void* const all[] = {(void*)k_implicit_dynamo<false, false, false>, (void*)k_implicit_dynamo<true, false, false>,
+                                   (void*)k_implicit_dynamo<false, false, true>, (void*)k_implicit_dynamo<true, false, true>,
+                                   (void*)k_implicit_dynamo<false, true, false>, (void*)k_implicit_dynamo<true, true, false>};
+        std::printf("%d\n", (int)(std::find(all, all + 6, fn) - all) + 1);
+    }
+}
+"""
+
+
+def test_dynamo_form_has_its_own_kernel(run):
+    """xi != 0 launches the kernel with the general solve inline, of the same variant; xi = 0 does not."""
+    rows = [[m, xi, acc, cc] for xi in (0.3, -1e-300, 0.0) for cc in (0, 1) for acc in (0, 1) for m in (0, 1)
+            if not (cc and acc)]
+    got = [r[0] for r in run(KERNELS, rows)]
+    assert got == [7 if xi == 0.0 else 1 + m + 2 * acc + 4 * cc for m, xi, acc, cc in rows]
 
 
 # the sources of a cell on a metric with psi alone
