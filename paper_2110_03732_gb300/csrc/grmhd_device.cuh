@@ -1394,7 +1394,12 @@ __device__ __forceinline__ bool newton_inverse_f32(const CellDW& c, const float*
 // error by ~1e-6 per step and the quadratic term is ~|dx|^2, so such a step (1e-9 at the
 // default tolerance) leaves ~1e-15 and the FP64 residual can accept it directly.  (Ending
 // at 3e-8 left up to 2e-14 in a cold first step; a start from the extrapolated history
-// takes as many evaluations either way.)  After a step |dx| <= 1e-5 max(|u|, 1) the next
+// takes as many evaluations either way.)  The step must also be small beside the momentum
+// scale, w_t |dx| <= 3e5 tol M (3e-8 M at the default tolerance, which leaves below 1e-14 M):
+// in a cell slower than 1e-9 every step is small beside 1, and the one step it took left a
+// residual that the FP64 test refused.  (Cells refused per solve and us per launch, steps 21
+// to 100: shock tube of 4096 cells 11, 31.7 -> 0, 14.8; telegraph 64 x 32 2047, 31.6 -> 0, 14.6;
+// 301^2 vortex 1, 42.5 -> 0, 28.5.)  After a step |dx| <= 1e-5 max(|u|, 1) the next
 // one reuses the inverse Jacobian: it has changed by that much, and the next step is that
 // much smaller again.  Steps are taken only when finite and within the step bound.
 //
@@ -1461,7 +1466,8 @@ __device__ __forceinline__ bool newton_refine_dw(const CellDW& c, dw* u, float t
         if (!(nx2 <= 1e4f * uu)) return false;   // also rejects NaN
 #pragma unroll
         for (int i = 0; i < 3; i++) u[i] = dw_add_f(u[i], dx[i]);
-        if (!ACC && (small || nx2 <= 1e-5f * tol * uu)) return false;
+        const float dm = fmaxf(fabsf(dx[0]), fmaxf(fabsf(dx[1]), fabsf(dx[2])));
+        if (!ACC && (small || (nx2 <= 1e-5f * tol * uu && dm * ed.wt <= 3e5f * tol * ed.M))) return false;
         reuse = nx2 <= 1e-10f * uu;
     }
     return false;

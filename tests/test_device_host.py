@@ -156,6 +156,18 @@ def test_cell_at_rest_takes_the_direct_path(run, a_dt):
         assert row[6] == 0
 
 
+@pytest.mark.parametrize("a_dt", [0.0, 0.05])
+@pytest.mark.parametrize("r", [0.0, 1e-6])
+def test_slow_cell_takes_the_direct_path(run, a_dt, r):
+    """The residual is measured by the cell's own momentum, so a start a few times off is corrected
+    to it on the direct path however slow the cell is.  (1e-12: ten times the tolerance; with
+    fields the momentum is their E x B, and that relative to it.)"""
+    for row in implicit(run, [[1.0, r * us, a_dt, us, 3 * us] for us in (1e-3, 1e-6, 1e-10, 1e-16, 1e-22)]):
+        assert row[0] == 0 and row[6] == 0
+        if a_dt == 0.0 or r == 0.0:
+            assert row[3] / row[2] == pytest.approx(-1.5, rel=1e-12) and row[4] / row[2] == pytest.approx(0.75, rel=1e-12)
+
+
 @pytest.mark.parametrize("acc", [False, True])
 @pytest.mark.parametrize("a_dt", [0.0, 0.05])
 def test_refused_cell_goes_on_from_the_corrections(run, a_dt, acc):
