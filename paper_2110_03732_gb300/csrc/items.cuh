@@ -188,6 +188,50 @@ __device__ __noinline__ void implicit_general(const Dims& g, const ImpArgs& a, l
     implicit_solve<M, CC, ACC>(g, a, t, refined, r0, r1, r2);
 }
 
+// A mixed-precision cell at rest (emode 0 or 1) whose start is u = 0, from its FP64 residual;
+// false where that does not vanish.  A short call: inline it cost the direct path of every
+// other cell (512^2 vortex 41 -> 43 us per launch), and the general solve costs such a cell more
+// (384^2 blast, cold, all but the edge at rest: 60 against 44).
+template <bool M, bool CC>
+__device__ __noinline__ bool implicit_rest(const Dims& g, const ImpArgs& a, long long t)
+{
+    int c[3];
+    interior_coords(g, t, c);
+    const long long id = lin(g, c[0], c[1], c[2]);
+    const double ps = M && a.psi ? a.psi[id] : 1.0, al = M && a.alp ? a.alp[id] : 1.0;
+    const double p2 = ps * ps, p4 = p2 * p2, ip2 = M ? rcp_pos(p2) : 1.0, ip4 = ip2 * ip2, ip6 = ip4 * ip2;
+    // W = 1, E = (eta_t E* / (1 + eta_t)) (E held fixed: E*), w_t = (tau + D - U - D / Gamma_hat)
+    // / (1 - 1 / Gamma_hat), and the residual is E x B - S
+    const double et = a.eta ? a.eta[id] : a.eta_u;
+    const double etat = M ? et * rcp_pos(al) * a.ia_dt : et * a.ia_dt;
+    const double k = a.stiff ? etat * rcp_wide(1.0 + etat) : 1.0;   // (NaN for an infinite eta_t)
+    double q[3], E[3], B[3], U2 = 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        q[i] = a.qb.p[5 + i][id];
+        E[i] = k * (q[i] * ip4);
+        B[i] = (CC ? a.bf.p[i][id] : cell_qB_in(g, a.bf.p[i], i, c, id)) * ip4;
+        U2 += E[i] * E[i] + B[i] * B[i];
+    }
+    bool zero = k >= 0.0 && (!a.stiff || etat >= 0.0);   // (a negative eta_t holds E fixed too)
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        const int j = (i + 1) % 3, l = (i + 2) % 3;
+        if (!(E[j] * B[l] - E[l] * B[j] == a.qb.p[1 + i][id] * ip6 * ip2)) zero = false;
+    }
+    const double rho = a.qb.p[0][id] * ip6;
+    const double wt = (a.qb.p[4][id] * ip6 + rho - 0.5 * U2 - rho * g.igh) * rcp_pos(1.0 - g.igh);
+    if (!zero || !pos_int(wt)) return false;
+    const double z[3] = {0.0, 0.0, 0.0}, pres = (wt - rho) * g.igh;
+    const float uh[3] = {0.0f, 0.0f, 0.0f};
+    float f32[11];
+    implicit_f32<M>(rho, pres, z, E, ip2, f32);
+#pragma unroll
+    for (int i = 0; i < 3; i++) f32[8 + i] = d2f_int(B[i] * p4);
+    implicit_store<M>(a, id, rho, pres, z, E, ip2, p4, q, f32, uh);
+    return true;
+}
+
 // the dynamo form (xi != 0), which has no direct path
 __device__ __forceinline__ bool has_dynamo(const ImpArgs& a) { return (__double_as_longlong(a.xi) << 1) != 0; }
 
@@ -282,7 +326,10 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
     float f32[11], uh[3];
     if (ACC) {
         if (!acc) {
-            implicit_general<M, CC, ACC>(g, a, t, ok, dw_to_double(ud[0]), dw_to_double(ud[1]), dw_to_double(ud[2]));
+            // (a momentum scale of zero: a cell at rest, and a start of zero)
+            const bool rest = ok && !(rt.M > 0.0f) && !((ud[0].hi != 0.0f) || (ud[1].hi != 0.0f) || (ud[2].hi != 0.0f));
+            if (!(rest && implicit_rest<M, CC>(g, a, t)))
+                implicit_general<M, CC, ACC>(g, a, t, ok, dw_to_double(ud[0]), dw_to_double(ud[1]), dw_to_double(ud[2]));
             return;
         }
         const double iW = dw_finite(dw_rcp(rt.W));

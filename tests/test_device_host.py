@@ -147,11 +147,12 @@ def test_implicit_solve_at_any_scale(run, a_dt):
         assert row[1:6] == pytest.approx(rows[0][1:6], rel=1e-11)
 
 
+@pytest.mark.parametrize("acc", [False, True])
 @pytest.mark.parametrize("a_dt", [0.0, 0.05])
-def test_cell_at_rest_takes_the_direct_path(run, a_dt):
+def test_cell_at_rest_takes_the_direct_path(run, a_dt, acc):
     """A cell without momentum has the momentum scale zero: its start u = 0 solves it exactly, and
     the direct path accepts that."""
-    for row in implicit(run, [[s, 0.0, a_dt, 0.0, 0.0] for s in (1.0, 1e-12, 1e6)]):
+    for row in implicit(run, [[s, 0.0, a_dt, 0.0, 0.0] for s in (1.0, 1e-12, 1e6)], acc):
         assert row[:1] + row[2:5] == [0.0] * 4 and row[1::4] == pytest.approx([1.3, 0.7], rel=1e-14)
         assert row[6] == 0
 
