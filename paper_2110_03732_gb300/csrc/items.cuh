@@ -13,18 +13,18 @@ namespace grmhd {
 // implicit step (Sec. 2.4): item t = interior cell t (x fastest)
 // ---------------------------------------------------------------------------
 
-// The outputs of a solved cell: primitives (FP64, and on the mixed path their FP32 copy
+// The outputs of a solved cell: primitives (FP64, and on the mixed path, F32, their FP32 copy
 // from the caller's f32 = rho, u^1..3, p, E^1..3, q_B^1..3), the stiff rate R, the solved
 // q_E and the history (uh: the FP32 orthonormal velocity, or NULL).  u and E orthonormal;
 // qEs the stage base's q_E.
-template <bool M>
+template <bool M, bool F32>
 __device__ __forceinline__ void implicit_store(const ImpArgs& a, long long id, double rho, double pres,
                                                const double* u, const double* E, double ip2, double p4,
                                                const double* qEs, const float* f32, const float* uh)
 {
     a.prim.p[0][id] = rho;
     a.prim.p[4][id] = pres;
-    if (a.p32.p[0]) {
+    if (F32 && a.p32.p[0]) {
 #pragma unroll
         for (int v = 0; v < 11; v++) a.p32.p[v][id] = f32[v];
     }
@@ -176,7 +176,7 @@ __device__ __forceinline__ void implicit_solve(const Dims& g, const ImpArgs& a, 
         f32[8 + i] = d2f_int(ci.B[i] * p4);
         uh[i] = d2f_int(u[i]);
     }
-    implicit_store<M>(a, id, rho, pres, u, e.E, ip2, p4, qEs, f32, atmo ? nullptr : uh);
+    implicit_store<M, ACC>(a, id, rho, pres, u, e.E, ip2, p4, qEs, f32, atmo ? nullptr : uh);
 }
 
 // the same as a call, so that its FP64 iteration takes neither registers nor
@@ -228,7 +228,7 @@ __device__ __noinline__ bool implicit_rest(const Dims& g, const ImpArgs& a, long
     implicit_f32<M>(rho, pres, z, E, ip2, f32);
 #pragma unroll
     for (int i = 0; i < 3; i++) f32[8 + i] = d2f_int(B[i] * p4);
-    implicit_store<M>(a, id, rho, pres, z, E, ip2, p4, q, f32, uh);
+    implicit_store<M, true>(a, id, rho, pres, z, E, ip2, p4, q, f32, uh);
     return true;
 }
 
@@ -269,12 +269,12 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
             q[i] = qE(i);
             Es[i] = mul(q[i], ip4);
         }
-        if (a.p32.p[0]) {
+        if (ACC) {
             implicit_f32<M>(a.rho_atm, a.p_atm, z, Es, ip2, f32);
 #pragma unroll
             for (int i = 0; i < 3; i++) f32[8 + i] = d2f_int(mul(mul(qB(i), ip4), p4));
         }
-        implicit_store<M>(a, id, a.rho_atm, a.p_atm, z, Es, ip2, p4, q, f32, nullptr);
+        implicit_store<M, ACC>(a, id, a.rho_atm, a.p_atm, z, Es, ip2, p4, q, f32, nullptr);
         return;
     }
     // the start: this stage's last root plus its last change, or the latest velocity
@@ -345,7 +345,7 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
         implicit_f32<M>(rho, pres, u, E, ip2, f32);
 #pragma unroll
         for (int i = 0; i < 3; i++) f32[8 + i] = M ? d2f_int(mul(mul(qB(i), ip4), p4)) : B32[i];
-        implicit_store<M>(a, id, rho, pres, u, E, ip2, p4, q, f32, uh);
+        implicit_store<M, ACC>(a, id, rho, pres, u, E, ip2, p4, q, f32, uh);
     } else {
         double S[3], Es[3], B[3];
         const double Dn = mul(a.qb.p[0][id], ip6);
@@ -369,7 +369,7 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
         const double rho = Dn * e.iW, pres = fma(e.wt, e.iW, -rho) * g.igh;
 #pragma unroll
         for (int i = 0; i < 3; i++) uh[i] = d2f_int(u[i]);
-        implicit_store<M>(a, id, rho, pres, u, e.E, ip2, p4, q, f32, uh);
+        implicit_store<M, ACC>(a, id, rho, pres, u, e.E, ip2, p4, q, f32, uh);
     }
 }
 

@@ -37,8 +37,8 @@ struct ImpArgs {
     int kmax;
     double tol, rho_atm, p_atm;
     float tolf;             // tol in FP32 (for the double-word corrections)
-    int dwacc;              // mixed precision (tol >= 1e-11): the double-word residual
-                            // accepts the root (the ACC instantiations)
+    int dwacc;              // mixed precision: the double-word residual accepts the root, and
+                            // p32 is written (the ACC instantiations)
     int stiff;              // a_dt > 0 (else E is held fixed)
     int atm;                // rho_atm > 0 (an atmosphere is set)
     double d_atm;           // 10 rho_atm: cells with D below it are atmosphere

@@ -59,9 +59,9 @@ Dims grid4()
 }
 """
 
-# a state in a flat cell and its solve from another start: prints the failures, rho, u and p, and
+# a state in a flat cell and its solve from another start: prints the failures, rho, u and p,
 # how often the general solve and the double-word corrections were entered (with
-# -finstrument-functions)
+# -finstrument-functions), and the FP32 copy
 IMPLICIT = GRID + r"""
 static int general, refine;
 #define HOOK extern "C" __attribute__((no_instrument_function)) void
@@ -113,16 +113,21 @@ int main() {
         a.tol = 1e-13;
         a.tolf = 1e-13f;
         a.nfail = &nfail;
+        static float f32[11][8];
+        for (int v = 0; v < 11; v++) {
+            a.p32.p[v] = f32[v];
+            f32[v][3] = -1.0f;
+        }
         if (ACC) {
-            static float f32[11][8];
-            for (int v = 0; v < 11; v++) a.p32.p[v] = f32[v];
             a.tol = 1e-10;
             a.tolf = 1e-10f;
         }
         general = refine = 0;
         implicit_item<false, false, ACC>(g, a, 1);
-        std::printf("%a %a %a %a %a %a %a %a\n", (double)nfail, A[11][3] / s, A[12][3], A[13][3], A[14][3], A[15][3] / s,
+        std::printf("%a %a %a %a %a %a %a %a ", (double)nfail, A[11][3] / s, A[12][3], A[13][3], A[14][3], A[15][3] / s,
                     (double)general, (double)refine);
+        for (int v = 0; v < 11; v++) std::printf("%a ", (double)f32[v][3]);
+        std::printf("\n");
     }
 }
 """
@@ -153,7 +158,7 @@ def test_cell_at_rest_takes_the_direct_path(run, a_dt, acc):
     """A cell without momentum has the momentum scale zero: its start u = 0 solves it exactly, and
     the direct path accepts that."""
     for row in implicit(run, [[s, 0.0, a_dt, 0.0, 0.0] for s in (1.0, 1e-12, 1e6)], acc):
-        assert row[:1] + row[2:5] == [0.0] * 4 and row[1::4] == pytest.approx([1.3, 0.7], rel=1e-14)
+        assert row[:1] + row[2:5] == [0.0] * 4 and [row[1], row[5]] == pytest.approx([1.3, 0.7], rel=1e-14)
         assert row[6] == 0
 
 
@@ -167,6 +172,17 @@ def test_slow_cell_takes_the_direct_path(run, a_dt, r):
         assert row[0] == 0 and row[6] == 0
         if a_dt == 0.0 or r == 0.0:
             assert row[3] / row[2] == pytest.approx(-1.5, rel=1e-12) and row[4] / row[2] == pytest.approx(0.75, rel=1e-12)
+
+
+@pytest.mark.parametrize("us,u0", [(1.0, 0.1), (0.0, 0.0), (20.0, 0.0)])
+def test_only_the_mixed_solve_writes_the_fp32_copy(run, us, u0):
+    """On the direct path, at rest and through the general solve: the rounded primitives and field
+    in mixed precision, nothing in FP64 (which has no such copy)."""
+    r = 0.0 if us == 0.0 else 1.0
+    assert implicit(run, [[1.0, r, 0.0, us, u0]])[0][8:] == [-1.0] * 11
+    row = implicit(run, [[1.0, r, 0.0, us, u0]], acc=True)[0]
+    want = row[1:6] + [0.5 * r, 0.2 * r, -0.3 * r, 0.6 * r, -0.8 * r, 0.5 * r]
+    assert row[8:] == [float(np.float32(x)) for x in want]
 
 
 @pytest.mark.parametrize("acc", [False, True])
