@@ -18,8 +18,9 @@
 // sign 2^5 above them, and what lies below the last place, 2^-56 of the larger of the two
 // others, is dropped; the FP64 sequence rounds their difference at 2^-54.  A slope of zero
 // returns the cell value itself.  PPM takes the FP64 sequence in a window wider than
-// kFxSpread.  A window with an infinity, a NaN or whose largest value is nonzero and below
-// 2^-943 takes the FP64 sequence too.
+// kFxSpread.  A window with an infinity, a NaN or whose largest value, the far neighbour
+// replaced, is nonzero and below 2^-943 takes the FP64 sequence too.  Denormals count as
+// zero: a cell that is zero like one of its neighbours is flat.
 #pragma once
 
 #include <stdint.h>
@@ -182,11 +183,11 @@ GRMHD_HD bool fx_mc_cell(double a, double b, double x, double& lo, double& hi)
     const unsigned top = fx_max(ea, fx_max(eb, ex));
     const unsigned la = fx_max(eb, ex) + (5u << 20), lx = fx_max(ea, eb) + (5u << 20);
     const unsigned fa = ea < la ? ea : la, f = ex < lx ? ex : lx;
-    const unsigned E = fx_max(fx_max(fa, f), fx_max(eb, kFxMinE));
+    const unsigned E0 = fx_max(fx_max(fa, f), eb), E = fx_max(E0, kFxMinE);
     const long long c = fx_cut(b, eb, E), h = fx_half_slope(fx_cut(a, fa, E), c, fx_cut(x, f, E));
     lo = h ? fx_to(c - h, E) : b;
     hi = h ? fx_to(c + h, E) : b;
-    return top - kFxMinE < 0x7ff00000u - kFxMinE || top == 0u;
+    return top < 0x7ff00000u && (E0 >= kFxMinE || (eb | (ea < ex ? ea : ex)) == 0u);
 }
 
 // PPM at cell a0 with the next two cells a1, x, the slope s0 of a0 and the interface value

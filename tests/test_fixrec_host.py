@@ -147,3 +147,26 @@ def test_ppm_cell(cells, kind):
         for got, want in ((lo, l), (hi, rr), (ins, fin), (s1, fs1)):
             assert abs(Fr(got) - want) <= abs(want) / 2 ** 53 + big
     assert used > 1000
+
+
+@pytest.mark.parametrize("far", [0.0, 1e-290, 1.0, -1e200])
+def test_mc_cell_of_tiny_values(cells, far):
+    """Where the two smaller values lie below 2^-943 the cell goes to the FP64 sequence, however
+    large the third is; so whatever is accepted keeps the bound of any window.  Denormals count
+    as zero: a cell of which one difference is then zero is flat, off by no more than 2^-1022."""
+    rng = random.Random(7)
+    tiny = [0.0, 5e-324, 1e-310, 3e-308, 1e-300, 2e-300, 1e-286]
+    rows = []
+    for _ in range(600):
+        w = [far, rng.choice([-1, 1]) * rng.choice(tiny), rng.choice([-1, 1]) * rng.choice(tiny)]
+        rng.shuffle(w)
+        rows.append(w)
+    for (a, b, x), (ok, (lo, hi, _, _)) in zip(rows, cells("m", rows)):
+        if not ok:
+            continue
+        fb = Fr(b)
+        h = half_slope(Fr(a), fb, Fr(x))
+        tol = Fr(4, 2 ** 53) * max(abs(fb), abs(h)) + Fr(1, 2 ** 1022)
+        assert abs(Fr(lo) - (fb - h)) <= tol and abs(Fr(hi) - (fb + h)) <= tol
+    flat = [[0.0, 0.0, far], [far, 0.0, 0.0], [0.0, 0.0, 0.0]]
+    assert cells("m", flat) == [(1, [0.0] * 4)] * 3
