@@ -1564,7 +1564,7 @@ __device__ __forceinline__ void cell_sources_f32(const Dims& g, const float* con
     }
 }
 
-template <bool M, bool F32 = false>
+template <bool M, bool F32 = false, bool ALL = false>
 __device__ __forceinline__ void update_item(const Dims& g, const UpdateArgs& a, long long t)
 {
     // flat metric: alpha = psi = 1 known at compile time
@@ -1590,9 +1590,8 @@ __device__ __forceinline__ void update_item(const Dims& g, const UpdateArgs& a, 
             // far below the FP32 fluxes' own error) and widened by one FP64 add, in place of two
             // FP64 instructions per flux.
             float src[8];
-            cell_sources_f32(g, a.p32, psi, alp, c, o, src);
-#pragma unroll
-            for (int v = 0; v < 8; v++) {
+            if (!ALL) cell_sources_f32(g, a.p32, psi, alp, c, o, src);
+            auto divergence = [&](int v) {
                 dw acc = dw_make(0.0f);
 #pragma unroll
                 for (int d = 0; d < 3; d++) {
@@ -1602,7 +1601,18 @@ __device__ __forceinline__ void update_item(const Dims& g, const UpdateArgs& a, 
                     const dw term = dw_mul(two_sum(Fv[chk(g, o + g.st[d])], -Fv[o]), h);
                     acc = d == 0 ? term : dw_add(acc, term);   // (direction 0 is always active)
                 }
-                double L = -dw_to_double(acc);
+                return acc;
+            };
+            // ALL: every variable's flux loads before the first store, which the compiler does
+            // not move loads across
+            dw all[8];
+#pragma unroll
+            for (int v = 0; v < 8; v++)
+                if (ALL) all[v] = divergence(v);
+            if (ALL) cell_sources_f32(g, a.p32, psi, alp, c, o, src);
+#pragma unroll
+            for (int v = 0; v < 8; v++) {
+                double L = -dw_to_double(ALL ? all[v] : divergence(v));
                 if (sourced(v)) L += f2d_int(src[v]);
                 out_value(a, v, o, L, v >= 5);
             }

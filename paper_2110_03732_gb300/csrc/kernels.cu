@@ -39,9 +39,17 @@ thread_local bool launch_overlap = false;
 // SM; one variable at a time, 90-240 B of spills): 512^2 40.0 against 46.4 at 8 to 12 blocks,
 // 96^3 star 166 against 199-214 (42 and 181 with all eight divergences held at once).  FP64:
 // seven blocks flat (512^2 55.7; 56.5 unbounded, 58.2 at eight), ten with a metric (128^3
-// 748; 778 at twelve, 760 at eight; 903 before the sources were collected).
-template <bool M, bool F32>
-__global__ void __launch_bounds__(128, F32 ? 16 : (M ? 10 : 7)) k_update(Dims g, UpdateArgs a)
+// 756; 786 at twelve, 768 at eight; 903 before the sources were collected).
+//
+// A grid that fits five blocks per SM waits for each variable's loads in turn, not for
+// registers: there the FP32-flux instances hold all eight divergences at once (96 registers,
+// ALL in update_item).  us per launch, one variable at a time / all at once: star 24^3 27.3 /
+// 24.9, 40^3 30.2 / 27.3, vortex 224^2 20.9 / 19.1, 96^2 19.9 / 19.5; 48^3 (5.7 blocks) 34.6 either
+// way.
+constexpr int kUpdateSmall = 5;   // blocks per SM of the ALL instances (launch_update)
+
+template <bool M, bool F32, bool ALL = false>
+__global__ void __launch_bounds__(128, ALL ? kUpdateSmall : (F32 ? 16 : (M ? 10 : 7))) k_update(Dims g, UpdateArgs a)
 {
     grid_dep_sync();
     long long tot = 1;
@@ -49,7 +57,7 @@ __global__ void __launch_bounds__(128, F32 ? 16 : (M ? 10 : 7)) k_update(Dims g,
     for (int d = 0; d < 3; d++) tot *= g.act[d] ? g.n[d] + 1 : 1;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot;
          t += (long long)gridDim.x * blockDim.x)
-        update_item<M, F32>(g, a, t);
+        update_item<M, F32, ALL>(g, a, t);
 }
 
 // ---------------------------------------------------------------------------
@@ -364,7 +372,9 @@ cudaError_t launch_update(const Dims& g, const UpdateArgs& a, int nsm, cudaStrea
     for (int d = 0; d < 3; d++) work *= g.act[d] ? g.n[d] + 1 : 1;
     const int b = grid_for(work, 128, nsm);
     const bool m = a.psi || a.alp;
-    if (a.f32) launch_k(m ? k_update<true, true> : k_update<false, true>, b, 128, st, g, a);
+    if (a.f32 && b <= nsm * kUpdateSmall)
+        launch_k(m ? k_update<true, true, true> : k_update<false, true, true>, b, 128, st, g, a);
+    else if (a.f32) launch_k(m ? k_update<true, true> : k_update<false, true>, b, 128, st, g, a);
     else launch_k(m ? k_update<true, false> : k_update<false, false>, b, 128, st, g, a);
     return cudaGetLastError();
 }
