@@ -80,16 +80,21 @@ constexpr int kMinItems = 128;   // smallest chunk of any candidate (scratch siz
 // batched kernels
 // ---------------------------------------------------------------------------
 
-// (64 registers, as k_implicit)
-template <bool M, bool ACC>
-__global__ void __launch_bounds__(256, 4) kb_implicit(const ProbStage* __restrict__ P, int s, int stage,
+// (64 registers; DYN: the problems with the dynamo form, with its solve inline as in
+// k_implicit_dynamo and as many registers as it takes.  A launch passes over the chunks of the
+// other kind, so that a problem runs the same kernel whatever else is in the batch.)
+template <bool M, bool ACC, bool DYN>
+__global__ void __launch_bounds__(256, DYN ? 1 : 4) kb_implicit(const ProbStage* __restrict__ P, int s, int stage,
                                                   const Chunk* __restrict__ ch, int nch)
 {
     for (int i = blockIdx.x; i < nch; i += gridDim.x) {
         const Chunk k = ch[i];
         const ProbStage& ps = P[k.prob * s + stage];
-        for (long long t = k.begin + threadIdx.x; t < k.end; t += blockDim.x)
-            implicit_item<M, false, ACC>(ps.g, ps.imp, t);
+        if (has_dynamo(ps.imp) != DYN) continue;
+        for (long long t = k.begin + threadIdx.x; t < k.end; t += blockDim.x) {
+            if (DYN) implicit_solve<M, false, ACC>(ps.g, ps.imp, t, false, 0.0, 0.0, 0.0);
+            else implicit_item<M, false, ACC>(ps.g, ps.imp, t);
+        }
     }
 }
 
@@ -339,6 +344,7 @@ struct grmhd_batch_s {
     Cfg cfg[WL_KINDS];
     int nsm;
     std::vector<int> fixed_probs;       // problems with FIXED boundaries
+    bool plain[2], dynamo[2];           // a problem (without, with a metric) has the plain, the dynamo form
     BarrierState* d_bar;                // persistent launch: grid barrier (device)
     double wait_limit_s;                // persistent launch: limit of each barrier wait
     int persist_blocks;                 // persistent launch: co-resident blocks (0: not yet known)
@@ -411,6 +417,17 @@ void fill_desc(grmhd_batch* b, int p, double dt)
     }
 }
 
+// which kernels of the implicit solve the descriptors need
+void find_dynamo(grmhd_batch* b)
+{
+    for (int m = 0; m < 2; m++) b->plain[m] = b->dynamo[m] = false;
+    for (int p = 0; p < b->n; p++) {
+        const int m = ctx_metric(b->ctx[p]) ? 1 : 0;
+        if (b->desc[(size_t)p * b->s].imp.xi != 0.0) b->dynamo[m] = true;
+        else b->plain[m] = true;
+    }
+}
+
 int grid_of(const grmhd_batch* b, int kind, int m)
 {
     return std::max(1, b->cnt[kind][m]);
@@ -426,13 +443,12 @@ cudaError_t launch_stage(grmhd_batch* b, int stage, cudaStream_t st, unsigned ma
         if (!(mask >> kind & 1u) || !b->cnt[kind][m]) continue;
         const Chunk* ch = b->d_chunks + b->off[kind][m];
         const int nch = b->cnt[kind][m], th = b->cfg[kind].threads, gr = grid_of(b, kind, m);
-        if (b->mixed) {
-            if (m) kb_implicit<true, true><<<gr, th, 0, st>>>(P, s, stage, ch, nch);
-            else kb_implicit<false, true><<<gr, th, 0, st>>>(P, s, stage, ch, nch);
-        } else {
-            if (m) kb_implicit<true, false><<<gr, th, 0, st>>>(P, s, stage, ch, nch);
-            else kb_implicit<false, false><<<gr, th, 0, st>>>(P, s, stage, ch, nch);
-        }
+#define KB_IMP(MM, ACC)                                                                        \
+    if (b->plain[MM]) kb_implicit<MM, ACC, false><<<gr, th, 0, st>>>(P, s, stage, ch, nch);    \
+    if (b->dynamo[MM]) kb_implicit<MM, ACC, true><<<gr, th, 0, st>>>(P, s, stage, ch, nch);
+        if (b->mixed) { if (m) { KB_IMP(true, true) } else { KB_IMP(false, true) } }
+        else { if (m) { KB_IMP(true, false) } else { KB_IMP(false, false) } }
+#undef KB_IMP
     }
     for (int d = 0; d < 3; d++)
         for (int m = 0; m < 2; m++) {
@@ -547,6 +563,7 @@ grmhd_status grmhd_batch_create(grmhd_ctx* const* ctxs, int n, void* scratch, si
         fill_desc(b, p, 0.0);
         if (ctx_any_fixed(ctxs[p])) b->fixed_probs.push_back(p);
     }
+    find_dynamo(b);
     s = build_lists(b, 0);
     if (s != GRMHD_OK) {
         delete b;
@@ -569,6 +586,7 @@ grmhd_status grmhd_batch_set_dt(grmhd_batch* b, const double* dt, grmhd_stream_t
         }
     }
     if (dirty) {
+        find_dynamo(b);
         cudaError_t e = cudaMemcpyAsync(b->d_desc, b->desc.data(), b->desc.size() * sizeof(ProbStage),
                                         cudaMemcpyHostToDevice, (cudaStream_t)stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)stream);

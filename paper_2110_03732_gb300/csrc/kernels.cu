@@ -39,7 +39,8 @@ thread_local bool launch_overlap = false;
 // SM; one variable at a time, 90-240 B of spills): 512^2 40.0 against 46.4 at 8 to 12 blocks,
 // 96^3 star 166 against 199-214 (42 and 181 with all eight divergences held at once).  FP64:
 // seven blocks flat (512^2 55.7; 56.5 unbounded, 58.2 at eight), ten with a metric (128^3
-// 756; 786 at twelve, 768 at eight; 903 before the sources were collected).
+// 748; 778 at twelve, 760 at eight; 903 before the sources were collected; at ten it is 756 with
+// the trace of the sources summed from its positive terms).
 //
 // A grid that fits five blocks per SM waits for each variable's loads in turn, not for
 // registers: there the FP32-flux instances hold all eight divergences at once (96 registers,
