@@ -42,8 +42,7 @@ __global__ void __launch_bounds__(128) k_emf_ideal(Dims g, EmfArgs<double> a, Vb
         emf_ideal_item<C, M>(g, prim, a.bf, a.psi, a.alp, vb.p, a.Eh, t);
 }
 
-// faces per thread by march_len (start-up: 3 cells for MC, 5 for PPM, each about a
-// fifth of a face's work)
+// faces per thread by march_len
 template <int D, bool M, bool P>
 static void flux_march_launch(const Dims& g, int nsm, cudaStream_t st, const FluxArgs<double>& a)
 {
@@ -57,7 +56,7 @@ static void flux_march_launch(const Dims& g, int nsm, cudaStream_t st, const Flu
             q = 1;
         nb_sm = q;
     }
-    const int K = march_len(g.n[D], other, nsm, nb_sm, P ? 1.0 : 0.6, NT);
+    const int K = march_len(g.n[D], other, nsm, nb_sm, Flux64<P, false>::C0, NT);
     Dims gl = g;
     set_march(gl, D, K);
     launch_k(k_flux_march<D, M, P>, grid_for((long long)gl.dq[D].d * other, NT, nsm), NT, st, gl, a);

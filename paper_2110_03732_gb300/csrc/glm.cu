@@ -165,7 +165,7 @@ static cudaError_t glm_flux_launch(const Dims& g, const GlmFluxArgs& a, int nsm,
         if (!g.act[d]) continue;
         const long long other = d == 0 ? (long long)g.n[1] * g.n[2]
                                        : (d == 1 ? (long long)g.n[0] * g.n[2] : (long long)g.n[0] * g.n[1]);
-        set_march(L.g[d], d, march_len(g.n[d], other, nsm, nb_sm, P ? 1.0 : 0.6, NT));
+        set_march(L.g[d], d, march_len(g.n[d], other, nsm, nb_sm, Flux64<P, true>::C0, NT));
         nb += glm_grid((long long)L.g[d].dq[d].d * other, NT, nsm);
     }
     L.b0[3] = nb;

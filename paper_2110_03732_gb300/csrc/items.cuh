@@ -737,6 +737,11 @@ struct Flux64 {
     static constexpr int SL = P ? 6 : 4;
     static constexpr int NT = P ? 64 : 128;
     static constexpr int SM = NV * SL * NT;        // at most 48 KB
+    // a march's start-up in faces (march_len): PPM reconstructs two cells before the first face
+    // and loads four, which are two faces' work here, where reconstruction bounds the kernel
+    // (at 1, as in FP32, star 96^3 took marches too short: 4.22 ms per launch, 3.70 at 2 or 3; 24^3
+    // to 64^3 and the 2-D vortices the same at 1, 2 and 3)
+    static constexpr double C0 = P ? 2.0 : 0.6;
 };
 
 // The FP64 fluxes of K consecutive d-faces per thread, marched along d; CC: the 12

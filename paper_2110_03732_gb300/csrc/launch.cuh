@@ -65,10 +65,9 @@ inline int grid_for(long long work, int threads, int nsm)
 // Items (faces or edges) per thread of a march over `other` lines of n + 1 items, with
 // blocks of `threads` of which bps are resident per SM: the K in 8..1 that minimises
 // (waves of resident blocks) x (K + c0), c0 being a march's start-up in items (the
-// cells reconstructed before the first item).  The kernels keep about two blocks per
-// SM and are latency- rather than throughput-limited at that occupancy, so an SM given
-// fewer blocks does not finish sooner: what counts is how many waves there are and how
-// long each thread's march is.  Ties go to the larger K (fewer loads and slopes).
+// cells reconstructed before the first item).  A wave of resident blocks takes as long as a
+// thread's march in it, whether or not it is full, so what counts is how many waves there are
+// and how long each march is.  Ties go to the larger K (fewer loads and slopes).
 inline int march_len(int n, long long other, int nsm, int bps, double c0, int threads = 128)
 {
     int best = 8;

@@ -142,7 +142,7 @@ cudaError_t stencil_launch(const Dims& g, const PrimIn<T>& prim, CP3 bf, const d
         nb_sm = q;
     }
     const int bps = nb_sm;
-    const double c0 = P ? 1.0 : 0.6;
+    const double c0 = sizeof(T) == 8 ? Flux64<P, false>::C0 : (P ? 1.0 : 0.6);
     StencilTasks<T> L;
     memset(&L, 0, sizeof L);
     int nb = 0;
