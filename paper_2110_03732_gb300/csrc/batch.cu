@@ -92,10 +92,18 @@ __global__ void __launch_bounds__(256, DYN ? 1 : 4) kb_implicit(const ProbStage*
         const ProbStage& ps = P[k.prob * s + stage];
         if (has_dynamo(ps.imp) != DYN) continue;
         for (long long t = k.begin + threadIdx.x; t < k.end; t += blockDim.x) {
-            if (DYN) implicit_solve<M, false, ACC>(ps.g, ps.imp, t, false, 0.0, 0.0, 0.0);
+            if (DYN) implicit_solve<M, false, ACC, true>(ps.g, ps.imp, t, false, 0.0, 0.0, 0.0);
             else implicit_item<M, false, ACC>(ps.g, ps.imp, t);
         }
     }
+}
+
+// either form, for the persistent launch
+template <bool M, bool ACC>
+__device__ __forceinline__ void implicit_any_item(const ProbStage& ps, long long t)
+{
+    if (has_dynamo(ps.imp)) implicit_general<M, false, ACC, true>(ps.g, ps.imp, t);
+    else implicit_item<M, false, ACC>(ps.g, ps.imp, t);
 }
 
 template <typename T> __device__ __forceinline__ const PrimIn<T>& prim_of(const ProbStage& ps);
@@ -277,8 +285,8 @@ __global__ void __launch_bounds__(128, (sizeof(T) == 4 ? 4 : 2)) kb_persistent(c
             if (!grid_barrier(bs, nb, limit_ns)) return;
         }
         for (int stage = 0; stage < s; stage++) {
-            PERSIST_ITEMS(WL_IMP, 0, (implicit_item<false, false, sizeof(T) == 4>(ps.g, ps.imp, t)))
-            PERSIST_ITEMS(WL_IMP, 1, (implicit_item<true, false, sizeof(T) == 4>(ps.g, ps.imp, t)))
+            PERSIST_ITEMS(WL_IMP, 0, (implicit_any_item<false, sizeof(T) == 4>(ps, t)))
+            PERSIST_ITEMS(WL_IMP, 1, (implicit_any_item<true, sizeof(T) == 4>(ps, t)))
             if (!grid_barrier(bs, nb, limit_ns)) return;
             PERSIST_ITEMS(WL_FLUX + 0, 0, (flux_any_item<0, false, T>(ps, sm, t)))
             PERSIST_ITEMS(WL_FLUX + 0, 1, (flux_any_item<0, true, T>(ps, sm, t)))

@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(128, CC ? 4 : 5) k_implicit_dynamo(const __gri
     const long long tot = (long long)g.n[0] * g.n[1] * g.n[2];
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot;
          t += (long long)gridDim.x * blockDim.x)
-        implicit_solve<M, CC, ACC>(g, a, t, false, 0.0, 0.0, 0.0);
+        implicit_solve<M, CC, ACC, true>(g, a, t, false, 0.0, 0.0, 0.0);
 }
 
 template <bool M, bool ACC>

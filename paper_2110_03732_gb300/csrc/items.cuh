@@ -63,8 +63,8 @@ __device__ __forceinline__ void implicit_f32(double rho, double pres, const doub
 // solve goes on from there (from its start where that is not finite) without repeating them.
 // CC: the magnetic field is cell-centred (a.bf holds cell q_B, GLM variant) instead of
 // staggered on faces.  ACC: the mixed-precision path, whose double-word residual
-// accepts the root (newton_refine_dw)
-template <bool M, bool CC, bool ACC>
+// accepts the root (newton_refine_dw).  DYN: the dynamo form may apply (xi != 0)
+template <bool M, bool CC, bool ACC, bool DYN>
 __device__ __forceinline__ void implicit_solve(const Dims& g, const ImpArgs& a, long long t, bool refined, double r0,
                                                double r1, double r2)
 {
@@ -88,7 +88,7 @@ __device__ __forceinline__ void implicit_solve(const Dims& g, const ImpArgs& a, 
     CellIn ci;
     ci.gh = g.gh;
     ci.igh = g.igh;
-    ci.xi = a.xi;
+    ci.xi = DYN ? a.xi : 0.0;
     ci.ighf = a.ighf;
     ci.xif = a.xif;
     ci.D = qb.p[0][id] * ip6;
@@ -135,10 +135,17 @@ __device__ __forceinline__ void implicit_solve(const Dims& g, const ImpArgs& a, 
             u[1] = r1;
             u[2] = r2;
         }
-        int it = newton_solve<ACC>(ci, u, e, kmax, tol, a.tolf, hist && fin, ust, refined);
-        if (it < 0 && fin) {
-            u[0] = u[1] = u[2] = 0.0;
-            it = newton_solve<ACC>(ci, u, e, kmax, tol, a.tolf, false, ust);
+        // from the start, then from rest.  One copy of the iteration where it is a call of the
+        // 72-register kernels (two spilled 1.8 KB, one 0.7 KB: 384^2 cold first solve on a metric
+        // 605 -> 580 us); with the registers of the dynamo kernels two are faster.
+        int it = -1;
+#pragma unroll(DYN ? 2 : 1)
+        for (int k = 0; k < 2; k++) {
+            if (k == 1) {
+                if (it >= 0 || !fin) break;
+                u[0] = u[1] = u[2] = 0.0;
+            }
+            it = newton_solve<ACC>(ci, u, e, kmax, tol, a.tolf, k == 0 && hist && fin, ust, k == 0 && refined);
         }
         if (it < 0) {
             atomicAdd(nfail, 1ull);
@@ -181,11 +188,11 @@ __device__ __forceinline__ void implicit_solve(const Dims& g, const ImpArgs& a, 
 
 // the same as a call, so that its FP64 iteration takes neither registers nor
 // instruction-cache room from the direct path
-template <bool M, bool CC, bool ACC>
+template <bool M, bool CC, bool ACC, bool DYN = false>
 __device__ __noinline__ void implicit_general(const Dims& g, const ImpArgs& a, long long t, bool refined = false,
                                               double r0 = 0.0, double r1 = 0.0, double r2 = 0.0)
 {
-    implicit_solve<M, CC, ACC>(g, a, t, refined, r0, r1, r2);
+    implicit_solve<M, CC, ACC, DYN>(g, a, t, refined, r0, r1, r2);
 }
 
 // A mixed-precision cell at rest (emode 0 or 1) whose start is u = 0, from its FP64 residual;
@@ -232,10 +239,11 @@ __device__ __noinline__ bool implicit_rest(const Dims& g, const ImpArgs& a, long
     return true;
 }
 
-// the dynamo form (xi != 0), which has no direct path
+// the dynamo form (xi != 0)
 __device__ __forceinline__ bool has_dynamo(const ImpArgs& a) { return (__double_as_longlong(a.xi) << 1) != 0; }
 
-// One cell: the direct path takes the double-word Newton corrections from the kept start
+// One cell (not of the dynamo form, which has no direct path: the callers take the general
+// solve there): the direct path takes the double-word Newton corrections from the kept start
 // and accepts their root by the FP64 residual (ACC: the double-word one); atmosphere cells
 // are written at once; everything else is implicit_general's.  The FP64 inputs are split
 // into double-words as they are loaded and loaded again for the FP64 residual (L1 holds
@@ -246,10 +254,6 @@ __device__ __forceinline__ void implicit_item(const Dims& g, const ImpArgs& a, l
     int c[3];
     interior_coords(g, t, c);
     const long long id = lin(g, c[0], c[1], c[2]);
-    if (has_dynamo(a)) {
-        implicit_general<M, CC, ACC>(g, a, t);
-        return;
-    }
     const double* __restrict__ psi = M ? a.psi : nullptr;
     const double* __restrict__ alp = M ? a.alp : nullptr;
     const double ps = psi ? psi[id] : 1.0;

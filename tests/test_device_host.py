@@ -68,7 +68,7 @@ static int general, refine;
 HOOK __cyg_profile_func_exit(void*, void*) {}
 HOOK __cyg_profile_func_enter(void* f, void*)
 {
-    general += f == (void*)implicit_general<false, false, ACC>;
+    general += f == (void*)implicit_general<false, false, ACC, false>;
     refine += f == (void*)newton_refine_dw<ACC>;
 }
 int main() {
