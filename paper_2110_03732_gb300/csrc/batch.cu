@@ -117,8 +117,7 @@ __device__ __forceinline__ FluxOut<float> flux32_of(const ProbStage& ps, int d)
     for (int v = 0; v < 8; v++) f.p[v] = reinterpret_cast<float*>(ps.F64[d].p[v]);
     return f;
 }
-// item t: kMarch consecutive D-faces
-// one item of either precision's face march
+// item t of either precision's face march: kMarch consecutive D-faces
 template <int D, bool M, typename T>
 __device__ __forceinline__ void flux_any_item(const ProbStage& ps, double* sm, long long t)
 {

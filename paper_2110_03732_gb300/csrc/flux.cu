@@ -69,14 +69,6 @@ static void flux_dispatch(const Dims& g, int d, bool m, int nsm, cudaStream_t st
     else m ? flux_march_launch<2, true, false>(g, nsm, st, a) : flux_march_launch<2, false, false>(g, nsm, st, a);
 }
 
-// edges of direction C (one per thread when A or B is inactive)
-static long long emf_work(const Dims& g, int c)
-{
-    long long work = 1;
-    for (int d = 0; d < 3; d++) work *= (d == c) ? g.n[d] : (g.act[d] ? g.n[d] + 1 : 1);
-    return work;
-}
-
 cudaError_t launch_flux(const Dims& g, int d, CP8 prim, CP3 bf, const double* psi, const double* alp, P8 F, int nsm,
                         cudaStream_t st, double* const* vbar, bool ppm, double* const* Eh)
 {

@@ -17,7 +17,7 @@
 // (d_t q + d_i f^i = s with the f_Phi and s_Phi of Sec. 3.1), which makes (B, Phi) a
 // damped wave system.  The charge field Psi is not evolved; rho_e comes from Gauss's
 // law as in the staggered scheme.  The implicit solve is the one of Sec. 2.4 with the
-// cell-centred field (k_implicit_cc in kernels.cu).
+// cell-centred field (k_implicit_cc in implicit.cu).
 #include "grmhd_device.cuh"
 #include "items.cuh"
 #include "kernels.h"
@@ -136,15 +136,6 @@ __global__ void __launch_bounds__(128) k_glm_update_metric(Dims g, GlmUpdateArgs
         glm_update_item<true>(g, a, t);
 }
 
-static int glm_grid(long long work, int threads, int nsm)
-{
-    long long b = (work + threads - 1) / threads;
-    const long long cap = (long long)nsm * 16;
-    if (b > cap) b = cap;
-    if (b < 1) b = 1;
-    return (int)b;
-}
-
 // faces per thread as for the staggered-field flux kernels
 template <bool M, bool P>
 static cudaError_t glm_flux_launch(const Dims& g, const GlmFluxArgs& a, int nsm, cudaStream_t st)
@@ -166,7 +157,7 @@ static cudaError_t glm_flux_launch(const Dims& g, const GlmFluxArgs& a, int nsm,
         const long long other = d == 0 ? (long long)g.n[1] * g.n[2]
                                        : (d == 1 ? (long long)g.n[0] * g.n[2] : (long long)g.n[0] * g.n[1]);
         set_march(L.g[d], d, march_len(g.n[d], other, nsm, nb_sm, Flux64<P, true>::C0, NT));
-        nb += glm_grid((long long)L.g[d].dq[d].d * other, NT, nsm);
+        nb += grid_for((long long)L.g[d].dq[d].d * other, NT, nsm);
     }
     L.b0[3] = nb;
     launch_k(k_glm_flux<M, P>, nb, NT, st, L);
@@ -182,7 +173,7 @@ cudaError_t launch_glm_flux(const Dims& g, const GlmFluxArgs& a, int nsm, cudaSt
 
 cudaError_t launch_glm_update(const Dims& g, const GlmUpdateArgs& a, int nsm, cudaStream_t st)
 {
-    const int b = glm_grid((long long)g.n[0] * g.n[1] * g.n[2], 128, nsm);
+    const int b = grid_for((long long)g.n[0] * g.n[1] * g.n[2], 128, nsm);
     launch_k(a.psi || a.alp ? k_glm_update_metric : k_glm_update_flat, b, 128, st, g, a);
     return cudaGetLastError();
 }

@@ -7,13 +7,14 @@
 
 namespace grmhd {
 
-// Seven blocks per SM (72 registers, 130-200 B of spills): the solve waits on its loads and
+// Seven blocks per SM (72 registers, 140-220 B of spills): the solve waits on its loads and
 // on dependent arithmetic, so more warps pay until the spills do not.  us per launch at
 // five / six / seven / eight blocks: 512^2 vortex FP64 65.7 / 61.7 / 60.3 / 61.2, mixed 44.6 /
 // 44.3 / 42.4 / 43.4; 96^3 star mixed 147 / 144 / 148 / 149.  (With the FP64 iteration inlined
 // in the kernel and the constants split at every residual it took 79.6 and 57.3 us at five
-// blocks, and 168 us; 128^3 star FP64 398 us, 277 now.)  The arguments are grid constants because implicit_general takes
-// them by reference: as plain parameters every thread copied them to its stack.
+// blocks, and 168 us; 128^3 star FP64 398 us, 280 now.)  The arguments are grid constants
+// because implicit_general takes them by reference: as plain parameters every thread copied
+// them to its stack.
 template <bool M, bool ACC>
 __global__ void __launch_bounds__(128, 7) k_implicit(const __grid_constant__ Dims g, const __grid_constant__ ImpArgs a)
 {
@@ -67,8 +68,9 @@ cudaError_t launch_implicit(const Dims& g, const ImpArgs& a, int nsm, cudaStream
 {
     const long long work = (long long)g.n[0] * g.n[1] * g.n[2];
     const bool m = a.psi || a.alp;
-    if (a.dwacc) launch_k(m ? implicit_kernel<true, true>(a) : implicit_kernel<false, true>(a), grid_for(work, 128, nsm), 128, st, g, a);
-    else launch_k(m ? implicit_kernel<true, false>(a) : implicit_kernel<false, false>(a), grid_for(work, 128, nsm), 128, st, g, a);
+    const int b = grid_for(work, 128, nsm);
+    if (a.dwacc) launch_k(m ? implicit_kernel<true, true>(a) : implicit_kernel<false, true>(a), b, 128, st, g, a);
+    else launch_k(m ? implicit_kernel<true, false>(a) : implicit_kernel<false, false>(a), b, 128, st, g, a);
     return cudaGetLastError();
 }
 

@@ -242,8 +242,8 @@ __device__ __noinline__ bool implicit_rest(const Dims& g, const ImpArgs& a, long
 // the dynamo form (xi != 0)
 __device__ __forceinline__ bool has_dynamo(const ImpArgs& a) { return (__double_as_longlong(a.xi) << 1) != 0; }
 
-// One cell (not of the dynamo form, which has no direct path: the callers take the general
-// solve there): the direct path takes the double-word Newton corrections from the kept start
+// One cell, not of the dynamo form (which has no direct path: the callers take the general
+// solve there).  The direct path takes the double-word Newton corrections from the kept start
 // and accepts their root by the FP64 residual (ACC: the double-word one); atmosphere cells
 // are written at once; everything else is implicit_general's.  The FP64 inputs are split
 // into double-words as they are loaded and loaded again for the FP64 residual (L1 holds
@@ -1688,6 +1688,14 @@ __device__ __forceinline__ void update_item(const Dims& g, const UpdateArgs& a, 
         if (g.act[fc]) r += (Eb[chk(g, o + g.st[fc])] - Eb[o]) * g.idx[fc];
         out_value(a, 8 + fa, o, r, false);
     }
+}
+
+// edges of direction C (one per thread when A or B is inactive)
+inline long long emf_work(const Dims& g, int c)
+{
+    long long work = 1;
+    for (int d = 0; d < 3; d++) work *= (d == c) ? g.n[d] : (g.act[d] ? g.n[d] + 1 : 1);
+    return work;
 }
 
 }  // namespace grmhd

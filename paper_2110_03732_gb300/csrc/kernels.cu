@@ -19,8 +19,8 @@
 //                (Sec. 3.2); writes L, or folds it straight into the IMEX stage bases and
 //                the final combination (Sec. 2.3)
 //   k_prim2con, k_curlA (Sec. 4), k_dt (Sec. 2.5), k_divb, k_totals: set-up and
-//   diagnostics; k_implicit_cc, k_curlA_cc, k_prim2con_cc, k_diag_cc: the same for the
-//   cell-centred fields of the GLM variant (its flux and update kernels: glm.cu)
+//   diagnostics; k_curlA_cc, k_prim2con_cc, k_diag_cc: the same for the cell-centred fields
+//   of the GLM variant (its flux and update kernels: glm.cu; k_implicit_cc: implicit.cu)
 #include "grmhd_device.cuh"
 #include "items.cuh"
 #include "kernels.h"

@@ -118,13 +118,6 @@ __global__ void __launch_bounds__(stencil_threads<T, P>(), sizeof(T) == 8 ? (P ?
     }
 }
 
-// edges of direction C (one per thread when A or B is inactive)
-static long long emf_work(const Dims& g, int c)
-{
-    long long work = 1;
-    for (int d = 0; d < 3; d++) work *= (d == c) ? g.n[d] : (g.act[d] ? g.n[d] + 1 : 1);
-    return work;
-}
 #endif
 
 // the launch of one instance: march lengths and block ranges of every task
